@@ -101,11 +101,74 @@ __device__ __forceinline__ uint4 pcg4d(uint4 v) {
 // conversion: the float with exponent 0 and mantissa m is 1 + m 2^-23, and
 // subtracting 1 - 2^-24 leaves (2m+1) 2^-24, which has at most 24 significant
 // bits and so is the exact difference (checked for every m).
+// (h >> 9) | 0x3F800000 is one funnel shift of the word pair (0x7F, h).
 __device__ __forceinline__ float hash_uniform(uint32_t h) {
-    return __fsub_rn(__uint_as_float((h >> 9) | 0x3F800000u), 0x1.fffffep-1f);
+    return __fsub_rn(__uint_as_float(__funnelshift_r(h, 0x7Fu, 9)), 0x1.fffffep-1f);
 }
 __device__ __forceinline__ float hash_uniform_complement(uint32_t h) {
     return __fsub_rn(1.f, hash_uniform(h));
+}
+
+// Packed FP32: two IEEE operations an instruction (sm_100 and later), each
+// rounded as its scalar form.  One takes two issue slots, as two scalar ones
+// do, and operands in adjacent registers: worth it where the pairs come that
+// way (texel channels, sibling nodes), not where they have to be assembled.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float lo2(f32x2 v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return a;
+}
+__device__ __forceinline__ float hi2(f32x2 v) {
+    float a, b;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    return b;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+// Four channels in two packed pairs, and acc + w t of them (w twice in w2).
+struct Quad {
+    f32x2 a, b;
+};
+__device__ __forceinline__ Quad fma4x2(f32x2 w2, const float4 &t, Quad acc) {
+    acc.a = fma2(w2, pack2(t.x, t.y), acc.a);
+    acc.b = fma2(w2, pack2(t.z, t.w), acc.b);
+    return acc;
+}
+__device__ __forceinline__ Quad fma4x2(f32x2 w2, const Quad &t, Quad acc) {
+    acc.a = fma2(w2, t.a, acc.a);
+    acc.b = fma2(w2, t.b, acc.b);
+    return acc;
+}
+
+// Two hash words' uniforms.
+__device__ __forceinline__ f32x2 hash_uniform2(uint32_t h1, uint32_t h2) {
+    return add2(pack2(__uint_as_float(__funnelshift_r(h1, 0x7Fu, 9)), __uint_as_float(__funnelshift_r(h2, 0x7Fu, 9))),
+                pack2(-0x1.fffffep-1f, -0x1.fffffep-1f));
 }
 
 // Equirect texel coordinates of a direction (texel centres at integers).
@@ -138,6 +201,9 @@ __device__ __forceinline__ Taps equirect_taps(float x, float y, int W, int H) {
     t.w10 = fy * (1.f - fx); t.w11 = fy * fx;
     return t;
 }
+
+// 2^e for -126 <= e <= 127.
+__device__ __forceinline__ float exp2_int(int e) { return __int_as_float((e + 127) << 23); }
 
 __device__ __forceinline__ float4 ldg4(const float4 *p) { return __ldg(p); }
 // Two float4 at a 32-byte aligned address in one 256-bit read-only load

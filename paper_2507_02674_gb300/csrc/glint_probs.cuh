@@ -147,11 +147,13 @@ __device__ __forceinline__ float4 lut_fetch(const float4 *lut, int n, float mu, 
     const int x0 = (int)fx0, y0 = (int)fy0;
     const int x1 = min(x0 + 1, n - 1), y1 = min(y0 + 1, n - 1);
     const float fx = x - fx0, fy = y - fy0;
-    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
-    r = fma4((1.f - fy) * (1.f - fx), __ldg(lut + y0 * n + x0), r);
-    r = fma4((1.f - fy) * fx, __ldg(lut + y0 * n + x1), r);
-    r = fma4(fy * (1.f - fx), __ldg(lut + y1 * n + x0), r);
-    r = fma4(fy * fx, __ldg(lut + y1 * n + x1), r);
+    Quad q{0, 0};
+    const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
+    q = fma4x2(pack2(w00, w00), __ldg(lut + y0 * n + x0), q);
+    q = fma4x2(pack2(w01, w01), __ldg(lut + y0 * n + x1), q);
+    q = fma4x2(pack2(w10, w10), __ldg(lut + y1 * n + x0), q);
+    q = fma4x2(pack2(w11, w11), __ldg(lut + y1 * n + x1), q);
+    const float4 r = make_float4(lo2(q.a), hi2(q.a), lo2(q.b), hi2(q.b));
     return r;
 }
 
@@ -172,9 +174,9 @@ template <int K, int C4, bool NEED_W>
 __device__ __forceinline__ void filtered_channels(const ShadeArgs &a, float th, float ph, int r0, int r1, float ft,
                                                   float *ch) {
     if (a.wfmt == GLINT_WFMT_F32) {
-        float4 cc[C4];
+        Quad cc[C4];
 #pragma unroll
-        for (int c = 0; c < C4; ++c) cc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c = 0; c < C4; ++c) cc[c] = Quad{0, 0};
 #pragma unroll
         for (int lv = 0; lv < 2; ++lv) {
             const int2 lev = __ldg(a.flev + (lv ? r1 : r0));
@@ -183,19 +185,22 @@ __device__ __forceinline__ void filtered_channels(const ShadeArgs &a, float th, 
             const float4 *base = a.filt + (size_t)lev.y * C4;
             const float wl = lv ? ft : 1.f - ft;
             constexpr int CN = NEED_W ? C4 : 1;
+            const f32x2 w00 = pack2(tp.w00, tp.w00), w01 = pack2(tp.w01, tp.w01), w10 = pack2(tp.w10, tp.w10),
+                        w11 = pack2(tp.w11, tp.w11), wl2 = pack2(wl, wl);
 #pragma unroll
             for (int c = 0; c < CN; ++c) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                v = fma4(tp.w00, __ldg(base + (size_t)tp.i00 * C4 + c), v);
-                v = fma4(tp.w01, __ldg(base + (size_t)tp.i01 * C4 + c), v);
-                v = fma4(tp.w10, __ldg(base + (size_t)tp.i10 * C4 + c), v);
-                v = fma4(tp.w11, __ldg(base + (size_t)tp.i11 * C4 + c), v);
-                cc[c] = fma4(wl, v, cc[c]);
+                Quad v{0, 0};
+                v = fma4x2(w00, __ldg(base + (size_t)tp.i00 * C4 + c), v);
+                v = fma4x2(w01, __ldg(base + (size_t)tp.i01 * C4 + c), v);
+                v = fma4x2(w10, __ldg(base + (size_t)tp.i10 * C4 + c), v);
+                v = fma4x2(w11, __ldg(base + (size_t)tp.i11 * C4 + c), v);
+                cc[c] = fma4x2(wl2, v, cc[c]);
             }
         }
 #pragma unroll
         for (int c = 0; c < C4; ++c) {
-            ch[4 * c] = cc[c].x; ch[4 * c + 1] = cc[c].y; ch[4 * c + 2] = cc[c].z; ch[4 * c + 3] = cc[c].w;
+            ch[4 * c] = lo2(cc[c].a); ch[4 * c + 1] = hi2(cc[c].a);
+            ch[4 * c + 2] = lo2(cc[c].b); ch[4 * c + 3] = hi2(cc[c].b);
         }
         return;
     }
@@ -349,9 +354,9 @@ template <int K>
 __device__ __forceinline__ void filtered_w(const ShadeArgs &a, float th, float ph, int r0, int r1, float ft,
                                            float *W) {
     constexpr int KW4 = (K + 3) / 4;
-    float4 cc[KW4];
+    Quad cc[KW4];
 #pragma unroll
-    for (int c = 0; c < KW4; ++c) cc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = 0; c < KW4; ++c) cc[c] = Quad{0, 0};
 #pragma unroll
     for (int lv = 0; lv < 2; ++lv) {
         const int2 lev = __ldg(a.flev + (lv ? r1 : r0));
@@ -359,38 +364,30 @@ __device__ __forceinline__ void filtered_w(const ShadeArgs &a, float th, float p
         const Taps tp = equirect_taps(ph * (kInvTwoPi * (float)Wr) - 0.5f, th * (kInvPi * (float)Hr) - 0.5f, Wr, Hr);
         const float4 *base = a.filtw + (size_t)lev.y * KW4;
         const float wl = lv ? ft : 1.f - ft;
-        if constexpr (KW4 == 2) {
-            // 32-byte texels in a cudaMalloc'd buffer: every texel is 32-byte aligned
-            float4 t[4][2];
-            ldg8(base + (size_t)tp.i00 * 2, t[0][0], t[0][1]);
-            ldg8(base + (size_t)tp.i01 * 2, t[1][0], t[1][1]);
-            ldg8(base + (size_t)tp.i10 * 2, t[2][0], t[2][1]);
-            ldg8(base + (size_t)tp.i11 * 2, t[3][0], t[3][1]);
+        float4 t[4][KW4];
+        const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
+        const float tw[4] = {tp.w00, tp.w01, tp.w10, tp.w11};
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                v = fma4(tp.w00, t[0][c], v);
-                v = fma4(tp.w01, t[1][c], v);
-                v = fma4(tp.w10, t[2][c], v);
-                v = fma4(tp.w11, t[3][c], v);
-                cc[c] = fma4(wl, v, cc[c]);
-            }
-        } else {
+        for (int j = 0; j < 4; ++j) {
+            if constexpr (KW4 == 2) {  // 32-byte texels in a cudaMalloc'd buffer: every texel is 32-byte aligned
+                ldg8(base + (size_t)idx[j] * 2, t[j][0], t[j][1]);
+            } else {
 #pragma unroll
-            for (int c = 0; c < KW4; ++c) {
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                v = fma4(tp.w00, __ldg(base + (size_t)tp.i00 * KW4 + c), v);
-                v = fma4(tp.w01, __ldg(base + (size_t)tp.i01 * KW4 + c), v);
-                v = fma4(tp.w10, __ldg(base + (size_t)tp.i10 * KW4 + c), v);
-                v = fma4(tp.w11, __ldg(base + (size_t)tp.i11 * KW4 + c), v);
-                cc[c] = fma4(wl, v, cc[c]);
+                for (int c = 0; c < KW4; ++c) t[j][c] = __ldg(base + (size_t)idx[j] * KW4 + c);
             }
+        }
+#pragma unroll
+        for (int c = 0; c < KW4; ++c) {
+            Quad v{0, 0};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v = fma4x2(pack2(tw[j], tw[j]), t[j][c], v);
+            cc[c] = fma4x2(pack2(wl, wl), v, cc[c]);
         }
     }
 #pragma unroll
     for (int k = 0; k < K; ++k) {
-        const float4 v = cc[k / 4];
-        W[k] = (k % 4 == 0) ? v.x : (k % 4 == 1) ? v.y : (k % 4 == 2) ? v.z : v.w;
+        const f32x2 v = (k & 2) ? cc[k / 4].b : cc[k / 4].a;
+        W[k] = (k & 1) ? hi2(v) : lo2(v);
     }
 }
 

@@ -21,9 +21,8 @@ namespace glint {
 
 __device__ __forceinline__ float normal_quantile(float p) {
     const float x = 2.f * p - 1.f;
-    const float p4 = 4.f * p;
     float w2;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(w2) : "f"(fmaf(-p4, p, p4)));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(w2) : "f"(fmaf(-x, x, 1.f)));
     w2 = -w2;
     float P;
     if (w2 < 7.213475227f) {
@@ -54,6 +53,45 @@ __device__ __forceinline__ float normal_quantile(float p) {
         P = fmaf(P, t, 4.006434441e+00f);
     }
     return P * x;
+}
+
+// normal_quantile of two arguments in packed FP32, the same results.  The tail
+// (0.35% of the uniforms) is evaluated for both when either needs it.
+__device__ __forceinline__ f32x2 normal_quantile2(f32x2 p) {
+    const f32x2 x = fma2(pack2(2.f, 2.f), p, pack2(-1.f, -1.f));
+    const f32x2 v = fma2(mul2(x, pack2(-1.f, -1.f)), x, pack2(1.f, 1.f));
+    float wa, wb;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(wa) : "f"(lo2(v)));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(wb) : "f"(hi2(v)));
+    const f32x2 t = sub2(pack2(-3.606737614f, -3.606737614f), pack2(wa, wb));
+    f32x2 P = pack2(-4.593011249e-10f, -4.593011249e-10f);
+    P = fma2(P, t, pack2(1.750330991e-09f, 1.750330991e-09f));
+    P = fma2(P, t, pack2(5.068341480e-08f, 5.068341480e-08f));
+    P = fma2(P, t, pack2(-5.430951546e-07f, -5.430951546e-07f));
+    P = fma2(P, t, pack2(-1.123125344e-06f, -1.123125344e-06f));
+    P = fma2(P, t, pack2(7.127850404e-05f, 7.127850404e-05f));
+    P = fma2(P, t, pack2(-5.900012329e-04f, -5.900012329e-04f));
+    P = fma2(P, t, pack2(-2.838380402e-03f, -2.838380402e-03f));
+    P = fma2(P, t, pack2(2.417711467e-01f, 2.417711467e-01f));
+    P = fma2(P, t, pack2(2.123313427e+00f, 2.123313427e+00f));
+    if (fminf(wa, wb) <= -7.213475227f) {
+        float ra, rb;
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(ra) : "f"(-wa));
+        asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(rb) : "f"(-wb));
+        const f32x2 s = add2(pack2(ra, rb), pack2(-3.603367329f, -3.603367329f));
+        f32x2 Q = pack2(3.712571197e-05f, 3.712571197e-05f);
+        Q = fma2(Q, s, pack2(-1.050955761e-04f, -1.050955761e-04f));
+        Q = fma2(Q, s, pack2(-3.455006663e-05f, -3.455006663e-05f));
+        Q = fma2(Q, s, pack2(7.061248762e-04f, 7.061248762e-04f));
+        Q = fma2(Q, s, pack2(-2.025795635e-03f, -2.025795635e-03f));
+        Q = fma2(Q, s, pack2(3.860775614e-03f, 3.860775614e-03f));
+        Q = fma2(Q, s, pack2(-6.235580891e-03f, -6.235580891e-03f));
+        Q = fma2(Q, s, pack2(9.259297512e-03f, 9.259297512e-03f));
+        Q = fma2(Q, s, pack2(1.179382324e+00f, 1.179382324e+00f));
+        Q = fma2(Q, s, pack2(4.006434441e+00f, 4.006434441e+00f));
+        P = pack2(wa <= -7.213475227f ? lo2(Q) : lo2(P), wb <= -7.213475227f ? hi2(Q) : hi2(P));
+    }
+    return mul2(P, x);
 }
 
 }  // namespace glint

@@ -17,7 +17,8 @@
 //      call, seed) give the uniforms (one call for the root's dither and node
 //      1, one per pair of sibling nodes), two hardware exp2 give the gate
 //      probabilities, and the Gaussian (normal quantile) is computed for every
-//      node, the gates selecting among the outcomes without branches;
+//      node, the gates selecting among the outcomes without branches; sibling
+//      nodes are drawn together in packed FP32;
 //   5. L^_o = L_o sum_k L_k M_k / (N_P sum_k L_k p_k).
 // 80 registers per thread (6 blocks of 128 threads per SM) measured fastest.
 #include "glint_shade_pixel.cuh"

@@ -54,6 +54,10 @@ __device__ __forceinline__ float fast_sqrt(float x) {
 struct NodeParams {
     float p, q, lp, lq;  // node probability, complement, log2 p, log2 of (1 - c p)^(1/c)
 };
+// The same of two sibling nodes, packed.
+struct NodePair {
+    f32x2 p, q, lp, lq;
+};
 
 // Dual-gated Gaussian (Alg. 1) for an integer number of trials N; returns n
 // (nbar = N - n), 0 when N = 0.  Regions of xi1 (same as the printed masks):
@@ -65,25 +69,55 @@ struct NodeParams {
 // Gaussian is computed for every lane and the gates select), so that a warp
 // whose lanes take different regions does not run the paths one after
 // another.  The Gaussian N(mu, sigma^2), mu = 1 + (N - 2) p, is rounded half
-// up as floor(sigma z + (mu + 1/2)).
+// up as floor(sigma z + (mu + 1/2)).  The small N need no cases of their own:
+// N = 1 takes p as its gate and leaves min(G, N - 1) = 0 below it; N = 0 has
+// P_{nbar=N} = exp2(0) = 1 (log2 q is kept finite), hence 0, and a NaN from
+// N - 2 < 0 under the root loses to 1 in the clamp.
 __device__ __forceinline__ uint32_t draw_integer(uint32_t N, const NodeParams &np, uint32_t h1, uint32_t h2) {
     const float xi1 = hash_uniform(h1);
-    const float xi1c = hash_uniform_complement(h1);
+    const float xi1c = __fsub_rn(1.f, xi1);
     const float Nf = __uint2float_rn(N);
-    const float m = fmaxf(Nf - 2.f, 0.f);  // N - 2 trials left to the Gaussian (0 below N = 2)
-    const float N2 = m + 2.f;
-    const bool many = N >= 2u;
-    const float Pall = many ? fast_exp2(N2 * np.lp) : 0.f;
-    const float T1 = many ? Pall : ((N == 1u) ? np.p : 0.f);
-    const float Sneg = fast_exp2(N2 * np.lq);  // decides only for N >= 2
+    const float m = Nf - 2.f;  // trials left to the Gaussian
+    const float T = (N == 1u) ? np.p : fast_exp2(Nf * np.lp);
+    const float Sneg = fast_exp2(Nf * np.lq);
     const float muh = fmaf(m, np.p, 1.5f);
     const float sigma = fast_sqrt(m * np.p * np.q);
     const float z = normal_quantile(hash_uniform(h2));
-    const float G = fminf(fmaxf(floorf(fmaf(sigma, z, muh)), 1.f), kMaxCount);
-    uint32_t r = min((uint32_t)G, N - 1u);
-    r = (xi1c <= Sneg || !many) ? 0u : r;
-    r = (xi1 < T1) ? 1u : r;
-    return (xi1 < Pall) ? N : r;
+    const float G = fmaxf(fmaf(sigma, z, muh), 1.f);
+    uint32_t r = min(__float2uint_rz(G), N - 1u);  // saturates above 2^32
+    r = (xi1c <= Sneg) ? 0u : r;
+    return (xi1 < T) ? N : r;
+}
+
+// draw_integer for two sibling nodes at once in packed FP32 (fma.rn.f32x2 and
+// its kin: two IEEE operations an instruction, the same results as one by
+// one).  h: the siblings' hash call, words (x, y) for the first, (z, w) for
+// the second.  The kernel is bound by issue slots.  A packed instruction takes
+// two of them, so the gain over two draw_integer calls is not the halved
+// arithmetic but one branch around the quantile's tail instead of two and
+// fewer, longer dependent chains: 126 cycles a pair against 142 (six resident
+// blocks of 128 threads).
+__device__ __forceinline__ void draw_integer_pair(uint32_t Na, uint32_t Nb, const NodePair &np, const uint4 &h,
+                                                  uint32_t &na, uint32_t &nb) {
+    const f32x2 xi1 = hash_uniform2(h.x, h.z);
+    const f32x2 xi1c = sub2(pack2(1.f, 1.f), xi1);
+    const f32x2 Nf = pack2(__uint2float_rn(Na), __uint2float_rn(Nb));
+    const f32x2 m = add2(Nf, pack2(-2.f, -2.f));
+    const f32x2 ea = mul2(Nf, np.lp), eb = mul2(Nf, np.lq);
+    const float Ta = (Na == 1u) ? lo2(np.p) : fast_exp2(lo2(ea));
+    const float Tb = (Nb == 1u) ? hi2(np.p) : fast_exp2(hi2(ea));
+    const float Sa = fast_exp2(lo2(eb)), Sb = fast_exp2(hi2(eb));
+    const f32x2 muh = fma2(m, np.p, pack2(1.5f, 1.5f));
+    const f32x2 var = mul2(mul2(m, np.p), np.q);
+    const f32x2 sigma = pack2(fast_sqrt(lo2(var)), fast_sqrt(hi2(var)));
+    const f32x2 z = normal_quantile2(hash_uniform2(h.y, h.w));
+    const f32x2 g = fma2(sigma, z, muh);
+    uint32_t ra = min(__float2uint_rz(fmaxf(lo2(g), 1.f)), Na - 1u);
+    uint32_t rb = min(__float2uint_rz(fmaxf(hi2(g), 1.f)), Nb - 1u);
+    ra = (lo2(xi1c) <= Sa) ? 0u : ra;
+    rb = (hi2(xi1c) <= Sb) ? 0u : rb;
+    na = (lo2(xi1) < Ta) ? Na : ra;
+    nb = (hi2(xi1) < Tb) ? Nb : rb;
 }
 
 // Dual-gated Gaussian (Alg. 1) with real-valued N and counts.
@@ -153,6 +187,33 @@ __device__ __forceinline__ NodeParams node_params(float pn, float qn) {
     nd.lp = l2p;
     nd.lq = (pn >= kEps) ? l2q : (pn * (1.f / kEps)) * kLog2OneMinusEps;
     return nd;
+}
+
+// log2 q made finite for draw_integer, whose N = 0 relies on 0 * log2 q = 0
+// (for N >= 1, N * -1e30 gives exp2 = 0 as -inf does).
+__device__ __forceinline__ float finite_log(float l) { return fminf(fmaxf(l, -1e30f), 1e30f); }
+
+// node_params of two sibling nodes, the series for log2(1 - x) in packed FP32
+// (the same operations, so the same values).
+__device__ __forceinline__ NodePair node_params2(float pa, float qa, float pb, float qb) {
+    constexpr float kTwoLog2e = 2.88539008177792681472f;
+    const bool la = pa <= 0.5f, lb = pb <= 0.5f;
+    const float xa = la ? pa : qa, xb = lb ? pb : qb;
+    const f32x2 s = pack2(__fdividef(xa, 2.f - xa), __fdividef(xb, 2.f - xb));
+    const f32x2 u = mul2(s, s);
+    f32x2 t = pack2(1.f / 13.f, 1.f / 13.f);
+    t = fma2(t, u, pack2(1.f / 11.f, 1.f / 11.f));
+    t = fma2(t, u, pack2(1.f / 9.f, 1.f / 9.f));
+    t = fma2(t, u, pack2(1.f / 7.f, 1.f / 7.f));
+    t = fma2(t, u, pack2(1.f / 5.f, 1.f / 5.f));
+    t = fma2(t, u, pack2(1.f / 3.f, 1.f / 3.f));
+    t = fma2(t, u, pack2(1.f, 1.f));
+    const f32x2 large = mul2(pack2(-kTwoLog2e, -kTwoLog2e), mul2(s, t));
+    const float sa = __log2f(xa), sb = __log2f(xb);
+    const float qla = la ? lo2(large) : sa, qlb = lb ? hi2(large) : sb;
+    return NodePair{pack2(pa, pb), pack2(qa, qb), pack2(la ? sa : lo2(large), lb ? sb : hi2(large)),
+                    pack2(finite_log((pa >= kEps) ? qla : (pa * (1.f / kEps)) * kLog2OneMinusEps),
+                          finite_log((pb >= kEps) ? qlb : (pb * (1.f / kEps)) * kLog2OneMinusEps))};
 }
 
 // Single-gated Gaussian for an integer number of trials N >= 1 (Sec. 5,
@@ -341,15 +402,30 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
 #pragma unroll
     for (int n = K - 1; n >= 1; --n) P[n] = P[2 * n] + P[2 * n + 1];
     NodeParams nd[K];
+    constexpr bool PAIRS = INTEGER && DRAW == kDrawDual;  // sibling nodes drawn two at a time
+    NodePair np2[K / 2];  // np2[m]: nodes 2m, 2m + 1
     if (DRAW == kDrawWang) {
         nd[1] = node_params(a.gamma, 1.f - a.gamma);
     } else {
+        float pn[K], qn[K];
 #pragma unroll
         for (int n = 1; n < K; ++n) {
             const float tot = P[n];
             const float inv = __fdividef(1.f, tot);  // hardware reciprocal, within 2 ulp
             const bool some = tot > 0.f;              // an empty subtree gets p = 0, q = 1
-            nd[n] = node_params(some ? P[2 * n] * inv : 0.f, some ? P[2 * n + 1] * inv : 1.f);
+            pn[n] = some ? P[2 * n] * inv : 0.f;
+            qn[n] = some ? P[2 * n + 1] * inv : 1.f;
+        }
+        nd[1] = node_params(pn[1], qn[1]);
+        if (PAIRS) nd[1].lq = finite_log(nd[1].lq);
+#pragma unroll
+        for (int m = 1; m < K / 2; ++m) {
+            if (PAIRS) {
+                np2[m] = node_params2(pn[2 * m], qn[2 * m], pn[2 * m + 1], qn[2 * m + 1]);
+            } else {
+                nd[2 * m] = node_params(pn[2 * m], qn[2 * m]);
+                nd[2 * m + 1] = node_params(pn[2 * m + 1], qn[2 * m + 1]);
+            }
         }
     }
 
@@ -376,14 +452,15 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
             const float cs = kOrientCos[o], sn = kOrientSin[o];
             const float up = __fadd_rn(__fmul_rn(cs, g2.x), __fmul_rn(sn, g2.y));
             const float vp = __fsub_rn(__fmul_rn(cs, g2.y), __fmul_rn(sn, g2.x));
-            x = ldexpf(up, -(l + an));
-            y = ldexpf(vp, -(l - an));
+            x = __fmul_rn(up, exp2_int(-(l + an)));  // exact scaling (l in [-24, 24], an in [0, 2])
+            y = __fmul_rn(vp, exp2_int(-(l - an)));
             key2 = (((uint32_t)l) & 0x3FFu) | ((uint32_t)an << 10) | ((uint32_t)o << 12) | 0x8000u;
         } else {
             l = l0 + lv;
             lw = lv ? fl : 1.f - fl;
-            x = ldexpf(g2.x, -l);
-            y = ldexpf(g2.y, -l);
+            const float scale = exp2_int(-l);  // exact scaling
+            x = __fmul_rn(g2.x, scale);
+            y = __fmul_rn(g2.y, scale);
             key2 = ((uint32_t)l) & 0xFFFFu;
         }
         const float sk = __fmul_rn(__fadd_rn(x, y), F2);
@@ -402,7 +479,7 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
             // the vertex's uniforms: hash call 1 gives the root's dither (word 0)
             // and node 1's pair (words 1, 2); siblings 2m, 2m+1 share call m + 1
             // (words 0, 1 and 2, 3), made once either of them has trials
-            uint4 h = pcg4d(make_uint4(vx, vy, key2 | (1u << 16), a.seed));
+            uint4 h = pcg4d(make_uint4(vx, vy, key2 + (1u << 16), a.seed));
             float cnt[K];
             float nroot;
             if (INTEGER) {
@@ -415,6 +492,21 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
                         N[K] = draw_single_integer(N[1], nd[1], h.y, h.z, false);
                         N[K + 1] = N[1] - N[K];
                     }
+                } else if (PAIRS) {
+                    N[2] = draw_integer(N[1], nd[1], h.y, h.z);
+                    N[3] = N[1] - N[2];
+#pragma unroll
+                    for (int m = 1; m < K / 2; ++m) {
+                        // a pair without trials in any lane of the warp is skipped (1080p, K = 8:
+                        // -0.5% of the frame; 3840 x 2160 grazing, K = 16: -2%)
+                        N[4 * m] = N[4 * m + 2] = 0u;
+                        if (N[2 * m] | N[2 * m + 1]) {
+                            h = pcg4d(make_uint4(vx, vy, key2 + ((uint32_t)(1 + m) << 16), a.seed));
+                            draw_integer_pair(N[2 * m], N[2 * m + 1], np2[m], h, N[4 * m], N[4 * m + 2]);
+                        }
+                        N[4 * m + 1] = N[2 * m] - N[4 * m];
+                        N[4 * m + 3] = N[2 * m + 1] - N[4 * m + 2];
+                    }
                 } else {
 #pragma unroll
                     for (int n = 1; n < K; ++n) {
@@ -423,12 +515,7 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
                             h = pcg4d(make_uint4(vx, vy, key2 | ((uint32_t)(1 + n / 2) << 16), a.seed));
                         const uint32_t u1 = (n == 1) ? h.y : (n & 1) ? h.z : h.x;
                         const uint32_t u2 = (n == 1) ? h.z : (n & 1) ? h.w : h.y;
-                        if (DRAW == kDrawDual) {
-                            // no branch: an empty node draws 0, and the
-                            // independent draws of sibling nodes interleave
-                            nl = draw_integer(N[n], nd[n], u1, u2);
-                            nr = N[n] - nl;
-                        } else if (N[n] > 0u) {
+                        if (N[n] > 0u) {
                             nl = draw_single_integer(N[n], nd[n], u1, u2, DRAW == kDrawSingleOld);
                             nr = N[n] - nl;
                         }
