@@ -345,7 +345,9 @@ glint_status glint_env_export(const glint_env *env, int item, int index, void *h
         float *dst = (float *)host_dst;
         for (size_t t = 0; t < texels; ++t) {
             memcpy(dst + t * env->C, rgb + 4 * t, sizeof(float) * 3);
-            memcpy(dst + t * env->C + 3, w + (size_t)4 * kw4 * t, sizeof(float) * d.K);
+            const int Wl = d.width >> index, x = (int)(t % Wl), y = (int)(t / Wl);
+            memcpy(dst + t * env->C + 3, w + (size_t)4 * kw4 * ((size_t)y * Wl + pyr_column(x, y, kw4)),
+                   sizeof(float) * d.K);
         }
         return GLINT_OK;
     }

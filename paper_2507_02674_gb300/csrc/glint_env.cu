@@ -142,12 +142,13 @@ __device__ __forceinline__ void texel_channels(float4 t, float scale, int K, con
     }
 }
 
-// Slot c of texel i of a pyramid level (float4 units of the split storage):
-// slot 0 is the colour (R, G, B, 0) at rgb4 + i, slots 1 .. C4-1 the weights
-// at w4 + i (C4 - 1) + c - 1.
+// Slot c of texel (x, y) of a pyramid level of width W (float4 units of the
+// split storage): slot 0 is the colour (R, G, B, 0) at rgb4 + y W + x, slots 1
+// .. C4-1 the weights at w4 + (y W + pyr_column(x, y, C4 - 1)) (C4 - 1) + c - 1.
 template <int C4>
-__device__ __forceinline__ size_t pyr_slot(size_t rgb4, size_t w4, size_t i, int c) {
-    return c == 0 ? rgb4 + i : w4 + i * (C4 - 1) + (c - 1);
+__device__ __forceinline__ size_t pyr_slot(size_t rgb4, size_t w4, int x, int y, int W, int c) {
+    const size_t row = (size_t)y * W;
+    return c == 0 ? rgb4 + row + x : w4 + (row + pyr_column(x, y, C4 - 1)) * (C4 - 1) + (c - 1);
 }
 
 // Steps 3 and 4: pyramid.  Each block takes a T x T tile of pyramid level m
@@ -188,11 +189,12 @@ __global__ void __launch_bounds__(kNT) k_pyramid(const void *__restrict__ texels
 #pragma unroll
             for (int c = 0; c < C4; ++c) {
                 v[c] = make_float4(tmp[4 * c], tmp[4 * c + 1], tmp[4 * c + 2], tmp[4 * c + 3]);
-                pyr[pyr_slot<C4>(rgb4[0], w4[0], gi, c)] = v[c];
+                pyr[pyr_slot<C4>(rgb4[0], w4[0], tx0 + lx, ty0 + ly, Ws, c)] = v[c];
             }
         } else {
 #pragma unroll
-            for (int c = 0; c < C4; ++c) v[c] = __ldcg(pyr + pyr_slot<C4>(rgb4[m], w4[m], gi, c));
+            for (int c = 0; c < C4; ++c)
+                v[c] = __ldcg(pyr + pyr_slot<C4>(rgb4[m], w4[m], tx0 + lx, ty0 + ly, Ws, c));
         }
     }
     __syncthreads();
@@ -224,7 +226,7 @@ __global__ void __launch_bounds__(kNT) k_pyramid(const void *__restrict__ texels
             r.z = (w0 * (a0.z + a1.z) + w1 * (b0.z + b1.z)) * inv;
             r.w = (w0 * (a0.w + a1.w) + w1 * (b0.w + b1.w)) * inv;
             bufB[t * C4 + c] = r;
-            pyr[pyr_slot<C4>(rgb4[m + l], w4[m + l], (size_t)(Y0 + y) * Wd + X0 + x, c)] = r;
+            pyr[pyr_slot<C4>(rgb4[m + l], w4[m + l], X0 + x, Y0 + y, Wd, c)] = r;
         }
         __syncthreads();  // (also: every store of the level issued before the block is counted as done)
         float4 *tmp = bufA;
@@ -251,17 +253,17 @@ __global__ void __launch_bounds__(kNT) k_pyramid(const void *__restrict__ texels
             const float w0 = sinf((2.f * Y + 0.5f) * (kPi / (float)Hc)) * sinf(half);
             const float w1 = sinf((2.f * Y + 1.5f) * (kPi / (float)Hc)) * sinf(half);
             const size_t r4 = rgb4[l - 1], ww4 = w4[l - 1];
-            const float4 a0 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, (size_t)(2 * Y) * Wc + 2 * x, c));
-            const float4 a1 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, (size_t)(2 * Y) * Wc + 2 * x + 1, c));
-            const float4 b0 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, (size_t)(2 * Y + 1) * Wc + 2 * x, c));
-            const float4 b1 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, (size_t)(2 * Y + 1) * Wc + 2 * x + 1, c));
+            const float4 a0 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x, 2 * Y, Wc, c));
+            const float4 a1 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x + 1, 2 * Y, Wc, c));
+            const float4 b0 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x, 2 * Y + 1, Wc, c));
+            const float4 b1 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x + 1, 2 * Y + 1, Wc, c));
             const float inv = 1.f / (2.f * (w0 + w1));
             float4 r;
             r.x = (w0 * (a0.x + a1.x) + w1 * (b0.x + b1.x)) * inv;
             r.y = (w0 * (a0.y + a1.y) + w1 * (b0.y + b1.y)) * inv;
             r.z = (w0 * (a0.z + a1.z) + w1 * (b0.z + b1.z)) * inv;
             r.w = (w0 * (a0.w + a1.w) + w1 * (b0.w + b1.w)) * inv;
-            pyr[pyr_slot<C4>(rgb4[l], w4[l], (size_t)Y * Wd + x, c)] = r;
+            pyr[pyr_slot<C4>(rgb4[l], w4[l], x, Y, Wd, c)] = r;
         }
         __syncthreads();  // level l complete before it is read
         Wc = Wd;
@@ -393,15 +395,18 @@ __global__ void __launch_bounds__(128) k_filter(const float4 *__restrict__ pyr, 
             const Taps tp = equirect_taps(xx, yy, Wm, Hm);
             const float4 *prgb = pyr + rgb4[m], *pw = pyr + w4[m];
             const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
+            // pyr_column of the weights
+            const int s0 = KW4 >= 2 && (tp.i00 & Wm) ? 2 : 0, s1 = KW4 >= 2 && (tp.i10 & Wm) ? 2 : 0;
+            const int widx[4] = {tp.i00 ^ s0, tp.i01 ^ s0, tp.i10 ^ s1, tp.i11 ^ s1};
             float4 tr[4], tw[4][KW4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 tr[j] = __ldg(prgb + idx[j]);
                 if constexpr (KW4 == 2) {
-                    ldg8(pw + (size_t)idx[j] * 2, tw[j][0], tw[j][1]);  // 32-byte aligned (even level offsets)
+                    ldg8(pw + (size_t)widx[j] * 2, tw[j][0], tw[j][1]);  // 32-byte aligned (even level offsets)
                 } else {
 #pragma unroll
-                    for (int c = 0; c < KW4; ++c) tw[j][c] = __ldg(pw + (size_t)idx[j] * KW4 + c);
+                    for (int c = 0; c < KW4; ++c) tw[j][c] = __ldg(pw + (size_t)widx[j] * KW4 + c);
                 }
             }
             float4 v = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -61,7 +61,7 @@ struct glint_env {
     float *pyr = nullptr;      // pyramid, all levels, Cpad floats per texel
     // Pyramid level m, in float4 units of `pyr`: its n_m texels' colour (R, G, B, 0)
     // at pyr_rgb4[m], then their weights W_1 .. W_K (Cpad/4 - 1 float4 per texel,
-    // zero past K) at pyr_w4[m] = pyr_rgb4[m] + n_m.  n_m is even, so at K = 8
+    // zero past K; columns as pyr_column has them) at pyr_w4[m] = pyr_rgb4[m] + n_m.  n_m is even, so at K = 8
     // every texel's 32 bytes of weights are 32-byte aligned.
     size_t pyr_rgb4[24] = {};
     size_t pyr_w4[24] = {};
@@ -120,13 +120,13 @@ __device__ __forceinline__ f32x2 pack2(float a, float b) {
     return r;
 }
 __device__ __forceinline__ float lo2(f32x2 v) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    float a;
+    asm("mov.b64 {%0, _}, %1;" : "=f"(a) : "l"(v));
     return a;
 }
 __device__ __forceinline__ float hi2(f32x2 v) {
-    float a, b;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+    float b;
+    asm("mov.b64 {_, %0}, %1;" : "=f"(b) : "l"(v));
     return b;
 }
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
@@ -202,6 +202,27 @@ __device__ __forceinline__ Taps equirect_taps(float x, float y, int W, int H) {
     return t;
 }
 
+// Column at which a pyramid level stores the weights of its texel (x, y), kw4
+// float4 each: from 32 bytes on (K >= 8) odd rows have the two halves of each
+// aligned four texels swapped.  The 2 x 2 texels of a bilinear look-up then lie
+// in four different 32-byte quarters of their 128-byte lines, wherever it
+// falls, and four lanes read them without a bank conflict (glint_e2.cu).
+// Smaller texels stay in order: they conflict less, and one thread that reads
+// all four pays for the swap (K = 2: 10% of the quadrature).  Levels with a
+// second row are at least four texels wide.
+__device__ __host__ __forceinline__ int pyr_column(int x, int y, int kw4) { return kw4 >= 2 ? x ^ ((y & 1) << 1) : x; }
+
+// equirect_taps with the columns of a pyramid level's weights.
+template <int KW4>
+__device__ __forceinline__ Taps pyr_weight_taps(float x, float y, int W, int H) {
+    Taps t = equirect_taps(x, y, W, H);
+    if (KW4 >= 2) {  // W is a power of two: the bit of an odd row
+        const int s0 = (t.i00 & W) ? 2 : 0, s1 = (t.i10 & W) ? 2 : 0;
+        t.i00 ^= s0; t.i01 ^= s0; t.i10 ^= s1; t.i11 ^= s1;
+    }
+    return t;
+}
+
 // 2^e for -126 <= e <= 127.
 __device__ __forceinline__ float exp2_int(int e) { return __int_as_float((e + 127) << 23); }
 
@@ -251,6 +272,8 @@ cudaError_t glint_launch_shade_variant(const glint::ShadeArgs &a, int K, bool in
 // kernel; p_k stays on chip).
 cudaError_t glint_launch_shade_mlp(const glint_ctx *ctx, const glint_env *env, const glint_gbuffer *g,
                                    const glint_params *p, float *out, const glint_debug *dbg, cudaStream_t s);
+// p_k of the E2 quadrature alone, a warp a pixel (glint_e2.cu).
+cudaError_t glint_launch_e2_probs(const glint::ShadeArgs &a, int K, int num_sms, cudaStream_t s);
 // p_k only (E1 or E2), background pixels 0.
 cudaError_t glint_launch_probs(const glint_ctx *ctx, const glint_env *env, const glint_gbuffer *g,
                                const glint_params *p, float *p_out, cudaStream_t s);

@@ -108,7 +108,7 @@ __device__ __forceinline__ void e2_probabilities(const ShadeArgs &a, long q, flo
             const float dx = c2 * hx - g0.x, dy = c2 * hy - g0.y, dz = c2 * hz - g0.z;
             float ex, ey;
             dir_to_texel(dx, dy, dz, Wm, Hm, ex, ey);
-            const Taps tp = equirect_taps(ex, ey, Wm, Hm);
+            const Taps tp = pyr_weight_taps<KW4>(ex, ey, Wm, Hm);
             float w[KW4 * 4];
             const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
             float4 tw[4][KW4];

@@ -142,12 +142,30 @@ cudaError_t glint_launch_shade(const glint_ctx *ctx, const glint_env *env, const
     return e;
 }
 
+// A warp a pixel (glint_e2.cu) or a thread a pixel for E2's p_k.  The warp's
+// points fill whole steps of 32 and pay for its set-up and final sums only from
+// some S on, sooner the more a point reads (1280 x 720, us, thread / warp; K = 2:
+// S = 14 1127 / 1223, S = 16 1467 / 1296, S = 24 3275 / 2905; K = 4: S = 16 1606 /
+// 1430; K = 8: S = 10 879 / 1000, S = 12 1280 / 1198, S = 32 9150 / 5780; K = 16:
+// S = 6 916 / 862, S = 16 7381 / 3230); steps are shorter where S is a power of
+// two.  Frames that leave most of the chip without a thread of its own take the
+// warp from S = 5 on (14400 pixels, S = 5: 22 / 14; 19200, K = 2, S = 4: 12 / 14;
+// 57600, S = 6: 35 / 50).
+static bool e2_by_warps(int K, int S, long npix, int num_sms) {
+    if (S >= 5 && npix <= 128L * num_sms) return true;
+    if (K == 16) return S >= 6;
+    if (K == 8) return S >= 12;
+    return S >= 24 || S == 16;
+}
+
 cudaError_t glint_launch_probs(const glint_ctx *ctx, const glint_env *env, const glint_gbuffer *g,
                                const glint_params *p, float *p_out, cudaStream_t s) {
     ShadeArgs a = make_args(ctx, env, g, p);
     a.p_out = p_out;
     const int ev = p->evaluator == GLINT_EVAL_E2 ? EV_E2 : p->evaluator == GLINT_EVAL_E1_ANISO ? EV_E1A : EV_E1;
     if (a.npix == 0) return cudaSuccess;
+    if (ev == EV_E2 && e2_by_warps(env->d.K, a.e2S, a.npix, ctx->num_sms))
+        return glint_launch_e2_probs(a, env->d.K, ctx->num_sms, s);
     switch (env->d.K) {
     case 2: return launch_probs<2>(a, ev, s);
     case 4: return launch_probs<4>(a, ev, s);
