@@ -152,6 +152,7 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
         sincospif(2.f * ((float)i + 0.5f) / (float)S, &sp, &cp);
         angle[i] = make_float2(cp, sp);
     }
+    pdl_wait_then_release();
     const long q0 = ((long)blockIdx.x * kWarps + warp) * ppw;
     if (lane < ppw) {
         E2Pixel e;
@@ -297,9 +298,7 @@ cudaError_t launch(const ShadeArgs &a, int num_sms, cudaStream_t s) {
     const long per_block = (long)kWarps * ppw;
     const unsigned grid = (unsigned)((a.npix + per_block - 1) / per_block);
     const bool fixed = a.e2S >= 8 && (a.e2S & (a.e2S - 1)) == 0;
-    if (fixed) k_e2_probs<K, true><<<grid, kWarps * 32, 0, s>>>(a, ppw);
-    else k_e2_probs<K, false><<<grid, kWarps * 32, 0, s>>>(a, ppw);
-    return cudaGetLastError();
+    return launch_pdl(true, fixed ? k_e2_probs<K, true> : k_e2_probs<K, false>, grid, kWarps * 32, 0, s, a, ppw);
 }
 
 }  // namespace

@@ -14,6 +14,8 @@
 // finished-block counter.
 #include <stdio.h>
 
+#include <algorithm>
+
 #include "glint_internal.cuh"
 
 using namespace glint;
@@ -56,7 +58,7 @@ __device__ void levels_from_partials(const float2 *partial, int nblk, int K, flo
     __shared__ float2 red[kNT / 32];
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(lo, hi);
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if ((int)threadIdx.x < K) {
         float mn = red[0].x, mx = red[0].y;
         for (int w = 1; w < kNT / 32; ++w) {
             mn = fminf(mn, red[w].x);
@@ -65,27 +67,65 @@ __device__ void levels_from_partials(const float2 *partial, int nblk, int K, flo
         lo = fmaxf(mn, ell);
         hi = fmaxf(mx, lo);
         const float l2 = log2f(hi / lo);
-        levels[0] = 0.f;
-        for (int k = 2; k <= K; ++k) {
-            const float a = (float)(k - 1) / (float)(K - 1);
-            levels[k - 1] = lo * exp2f(a * l2);
+        const int k = (int)threadIdx.x + 1;
+        const float a = (float)(k - 1) / (float)(K - 1);
+        levels[k - 1] = k == 1 ? 0.f : lo * exp2f(a * l2);
+        if (k == 1) {
+            levels[K] = lo;
+            levels[K + 1] = hi;
         }
-        levels[K] = lo;
-        levels[K + 1] = hi;
+    }
+}
+
+// Two adjacent texels 2 i, 2 i + 1 in 16-byte loads (16-byte aligned texels).
+__device__ __forceinline__ void load_texel_pair(const void *texels, int fmt, long i, float4 &a, float4 &b) {
+    if (fmt == GLINT_FMT_RGBA16F) {
+        const uint4 raw = __ldg(reinterpret_cast<const uint4 *>(texels) + i);
+        const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
+        const float2 f0 = __half22float2(h[0]), f1 = __half22float2(h[1]), f2 = __half22float2(h[2]),
+                     f3 = __half22float2(h[3]);
+        a = make_float4(f0.x, f0.y, f1.x, f1.y);
+        b = make_float4(f2.x, f2.y, f3.x, f3.y);
+    } else {
+        a = __ldg(reinterpret_cast<const float4 *>(texels) + 2 * i);
+        b = __ldg(reinterpret_cast<const float4 *>(texels) + 2 * i + 1);
     }
 }
 
 // Steps 1 and 2: per-block min / max of the brightness into the scratch
 // array; the last block to finish (counted in *done, which it resets) turns
-// the pairs into the levels.
+// the pairs into the levels, a thread a level.  Latency-bound (the map is a few
+// microseconds of HBM traffic): kMinMaxPairs independent loads of two texels a
+// thread.  wide: the texels are 16-byte aligned (n is even, a map being twice as
+// wide as high).
+constexpr int kMinMaxPairs = 4;
 __global__ void __launch_bounds__(kNT) k_minmax(const void *__restrict__ texels, int fmt, long n, float scale,
                                                   float2 *__restrict__ partial, unsigned *__restrict__ done, int K,
-                                                  float ell, float *__restrict__ levels) {
+                                                  float ell, float *__restrict__ levels, bool wide) {
+    pdl_release();
     float lo = INFINITY, hi = -INFINITY;
-    for (long i = (long)blockIdx.x * kNT + threadIdx.x; i < n; i += (long)gridDim.x * kNT) {
-        const float y = brightness(load_texel(texels, fmt, i), scale);
-        lo = fminf(lo, y);
-        hi = fmaxf(hi, y);
+    if (wide) {
+        for (long i0 = (long)blockIdx.x * (kNT * kMinMaxPairs) + threadIdx.x; i0 < n / 2;
+             i0 += (long)gridDim.x * (kNT * kMinMaxPairs)) {
+            float4 t[2 * kMinMaxPairs];
+#pragma unroll
+            for (int j = 0; j < kMinMaxPairs; ++j) {  // past the end: the first pair once more
+                const long i = i0 + j * kNT;
+                load_texel_pair(texels, fmt, i < n / 2 ? i : i0, t[2 * j], t[2 * j + 1]);
+            }
+#pragma unroll
+            for (int j = 0; j < 2 * kMinMaxPairs; ++j) {
+                const float y = brightness(t[j], scale);
+                lo = fminf(lo, y);
+                hi = fmaxf(hi, y);
+            }
+        }
+    } else {
+        for (long i = (long)blockIdx.x * kNT + threadIdx.x; i < n; i += (long)gridDim.x * kNT) {
+            const float y = brightness(load_texel(texels, fmt, i), scale);
+            lo = fminf(lo, y);
+            hi = fmaxf(hi, y);
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
@@ -114,13 +154,23 @@ __global__ void __launch_bounds__(kNT) k_minmax(const void *__restrict__ texels,
     if (threadIdx.x == 0) *done = 0u;
 }
 
-// Channel vector of one texel in the pyramid's slot order (R, G, B, 0,
-// w_1 .. w_K, 0 padding; Cpad floats): the fuzzy weights of the two levels
-// bracketing its brightness (Eq. wkdefpractice).
-__device__ __forceinline__ void texel_channels(float4 t, float scale, int K, const float *L, int Cpad, bool log_w,
-                                               float *v) {
-    const float R = t.x * scale, G = t.y * scale, B = t.z * scale;
-    const float Y = fmaxf(0.2126f * R + 0.7152f * G + 0.0722f * B, 0.f);
+// One texel's channels in the pyramid's slot order (R, G, B, 0, w_1 .. w_K, 0
+// padding): its colour and the fuzzy weights of the two levels bracketing its
+// brightness (Eq. wkdefpractice).
+struct TexelChannels {
+    float R, G, B;
+    int j;         // w_{j+1} = wa, w_{j+2} = wb, the others 0
+    float wa, wb;
+    __device__ __forceinline__ float weight(int k) const { return k == j ? wa : k == j + 1 ? wb : 0.f; }
+    __device__ __forceinline__ float4 slot(int c) const {
+        return c == 0 ? make_float4(R, G, B, 0.f)
+                      : make_float4(weight(4 * c - 4), weight(4 * c - 3), weight(4 * c - 2), weight(4 * c - 1));
+    }
+};
+__device__ __forceinline__ TexelChannels texel_channels(float4 t, float scale, int K, const float *L, bool log_w) {
+    TexelChannels o;
+    o.R = t.x * scale; o.G = t.y * scale; o.B = t.z * scale;
+    const float Y = fmaxf(0.2126f * o.R + 0.7152f * o.G + 0.0722f * o.B, 0.f);
     // bracket: largest j in [0, K-2] with L[j] <= Y; Y >= L[K-1] -> w_K = 1
     int j = 0;
     for (int k = 1; k < K - 1; ++k)
@@ -129,17 +179,10 @@ __device__ __forceinline__ void texel_channels(float4 t, float scale, int K, con
     // log space (optional, Sec. 7): between L_j > 0 and L_{j+1}; linear below L_2 (L_1 = 0)
     const float tt = (log_w && j > 0) ? (logf(Y) - logf(L[j])) / (logf(L[j + 1]) - logf(L[j]))
                                       : (Y - L[j]) / (L[j + 1] - L[j]);
-    v[0] = R; v[1] = G; v[2] = B; v[3] = 0.f;
-    for (int c = 4; c < Cpad; ++c) {
-        const int k = c - 4;
-        float val = 0.f;
-        if (k < K) {
-            if (top) val = (k == K - 1) ? 1.f : 0.f;
-            else if (k == j) val = 1.f - tt;
-            else if (k == j + 1) val = tt;
-        }
-        v[c] = val;
-    }
+    o.j = top ? K - 2 : j;
+    o.wa = top ? 0.f : 1.f - tt;
+    o.wb = top ? 1.f : tt;
+    return o;
 }
 
 // Slot c of texel (x, y) of a pyramid level of width W (float4 units of the
@@ -151,82 +194,150 @@ __device__ __forceinline__ size_t pyr_slot(size_t rgb4, size_t w4, int x, int y,
     return c == 0 ? rgb4 + row + x : w4 + (row + pyr_column(x, y, C4 - 1)) * (C4 - 1) + (c - 1);
 }
 
-// Steps 3 and 4: pyramid.  Each block takes a T x T tile of pyramid level m
-// (T <= 32, a power of two), writes it (for m = 0 computing the channels of the
-// texels first) and reduces it through log2 T further levels in shared memory,
-// writing each.  A texel of level l+1 is the solid-angle weighted mean of its
-// 2 x 2 children; the weight of a row spanning [theta0, theta1] is
-// cos theta0 - cos theta1 = 2 sin(mid) sin(half), written as a product to stay
-// accurate near the poles.  With tail_to > m + nlev the last block to finish
-// (counted in *done, which it resets) builds levels m + nlev + 1 .. tail_to
-// from level m + nlev, which every block has written by then.
+// Row weights of a level built from a parent of height Hp: of the two parent
+// rows under row Y and the reciprocal of their sum over the 2 x 2 children.  A
+// row spanning [theta0, theta1] weighs cos theta0 - cos theta1 = 2 sin(mid)
+// sin(half), written as a product to stay accurate near the poles.
+__device__ __forceinline__ float3 row_weights(int Y, int Hp) {
+    const float half = 0.5f * kPi / (float)Hp;
+    const float w0 = sinf((2.f * Y + 0.5f) * (kPi / (float)Hp)) * sinf(half);
+    const float w1 = sinf((2.f * Y + 1.5f) * (kPi / (float)Hp)) * sinf(half);
+    return make_float3(w0, w1, 1.f / (2.f * (w0 + w1)));
+}
+
+// Solid-angle weighted mean of the 2 x 2 children a0 a1 / b0 b1.
+__device__ __forceinline__ float mean4(float a0, float a1, float b0, float b1, float w0, float w1, float inv) {
+    return (w0 * (a0 + a1) + w1 * (b0 + b1)) * inv;
+}
+__device__ __forceinline__ float4 mean4(const float4 &a0, const float4 &a1, const float4 &b0, const float4 &b1,
+                                        const float3 &w) {
+    return make_float4(mean4(a0.x, a1.x, b0.x, b1.x, w.x, w.y, w.z), mean4(a0.y, a1.y, b0.y, b1.y, w.x, w.y, w.z),
+                       mean4(a0.z, a1.z, b0.z, b1.z, w.x, w.y, w.z), mean4(a0.w, a1.w, b0.w, b1.w, w.x, w.y, w.z));
+}
+
+// Steps 3 and 4: pyramid.  A block takes a 32 x 32 tile (T, a power of two; less
+// on maps below 32 rows) of pyramid level m and builds log2 T further levels.
+// Each thread holds a 2 x 2 quad of the tile in registers, writes it if the
+// texels' channels are computed here (m = 0), and writes the quad's mean, level
+// m + 1, to memory and to shared memory, where the upper levels are reduced.
+// (With the whole tile staged in shared memory, 60 KB a block at K = 8, only
+// three blocks fit an SM, 456 of the 512 of a 1024 x 512 map: two waves.)
+// Latency bounds it at small maps, so the row weights of all levels are computed
+// at the start and the texels fetched before the wait for the levels; at large
+// ones the stores, so they are whole 32-byte sectors a thread (16-byte pieces of
+// two texels a thread left half-written sectors).  1024 x 512, K = 8: 25.8 ->
+// 17.4 us; 2048 x 1024, K = 16 (223 MB written): 111 -> 75 us.  With tail_to > m + nlev the last block to finish
+// (counted in *done, which it resets) builds levels m + nlev + 1 .. tail_to from
+// level m + nlev, which every block has written by then: the first from memory,
+// the others from shared memory (at most kPyrTailTexels / 4 texels).
+constexpr long kPyrTailTexels = 2048;
+
+template <int C4>
+constexpr size_t pyramid_smem() {  // level m + 1 of a tile (256 texels) and m + 2, or the first two tail levels
+    return sizeof(float4) * C4 * (kPyrTailTexels / 4 + kPyrTailTexels / 16);
+}
+
 template <bool FROM_TEXELS, int C4>
-__global__ void __launch_bounds__(kNT) k_pyramid(const void *__restrict__ texels, int fmt, float scale, int K,
-                                                   const float *__restrict__ levels, float4 *__restrict__ pyr,
-                                                   const size_t *__restrict__ rgb4, const size_t *__restrict__ w4,
-                                                   int m, int Ws, int Hs, int T, int nlev, int log_w, int tail_to,
-                                                   unsigned *__restrict__ done) {
-    constexpr int Cpad = 4 * C4;
+__global__ void __launch_bounds__(kNT, 4) k_pyramid(
+    const void *__restrict__ texels, int fmt, float scale, int K, const float *__restrict__ levels,
+    float4 *__restrict__ pyr, const size_t *__restrict__ rgb4, const size_t *__restrict__ w4, int m, int Ws, int Hs,
+    int T, int nlev, int log_w, int tail_to, unsigned *__restrict__ done, bool wide) {
     extern __shared__ float4 smem4[];
-    float4 *bufA = smem4;                        // T*T texels of C4 float4
-    float4 *bufB = smem4 + (size_t)T * T * C4;   // (T/2)^2 texels
     __shared__ float L[GLINT_MAX_K];
-    __shared__ float4 rw[16];  // per row of the level being built: w0, w1, 1 / (2 (w0 + w1))
-    if (FROM_TEXELS) {
-        if (threadIdx.x < K) L[threadIdx.x] = levels[threadIdx.x];
-        __syncthreads();
-    }
+    __shared__ float3 rw[32];  // rows of levels m + 1, m + 2, ..: T/2, T/4, .., 1 of them
     // T is a power of two (2^nlev): tile coordinates by shifts and masks
     const int tiles_x = Ws >> nlev;
     const int tx0 = ((int)blockIdx.x & (tiles_x - 1)) << nlev, ty0 = ((int)blockIdx.x / tiles_x) << nlev;
-    for (int i = threadIdx.x; i < T * T; i += kNT) {
-        const int lx = i & (T - 1), ly = i >> nlev;
-        const size_t gi = (size_t)(ty0 + ly) * Ws + (tx0 + lx);
-        float4 *v = bufA + (size_t)i * C4;
-        if (FROM_TEXELS) {
-            float tmp[3 + GLINT_MAX_K + 1];
-            texel_channels(load_texel(texels, fmt, (long)gi), scale, K, L, Cpad, log_w != 0, tmp);
+    {
+        const int i = (int)threadIdx.x - (kNT - 32);  // the last warp
+        if (i >= 0 && i < T - 1) {
+            int l = 1, first = 0;
+            while (i >= first + (T >> l)) first += T >> l++;
+            rw[i] = row_weights((ty0 >> l) + i - first, Hs >> (l - 1));
+        }
+    }
+    // The first quad's texels are fetched before the wait on the kernel that finds
+    // the levels (which waited for whatever wrote them).
+    float4 tex[4] = {};
+    const int cur0 = T / 2;
+    if (FROM_TEXELS && (int)threadIdx.x < cur0 * cur0) {
+        const int x = threadIdx.x & (cur0 - 1), y = threadIdx.x >> (nlev - 1);
 #pragma unroll
-            for (int c = 0; c < C4; ++c) {
-                v[c] = make_float4(tmp[4 * c], tmp[4 * c + 1], tmp[4 * c + 2], tmp[4 * c + 3]);
-                pyr[pyr_slot<C4>(rgb4[0], w4[0], tx0 + lx, ty0 + ly, Ws, c)] = v[c];
+        for (int r = 0; r < 2; ++r) {
+            const long g = (long)(ty0 + 2 * y + r) * Ws + tx0 + 2 * x;
+            if (wide) {
+                load_texel_pair(texels, fmt, g / 2, tex[2 * r], tex[2 * r + 1]);
+            } else {
+                tex[2 * r] = load_texel(texels, fmt, g);
+                tex[2 * r + 1] = load_texel(texels, fmt, g + 1);
             }
+        }
+    }
+    pdl_wait_then_release();
+    if (FROM_TEXELS && threadIdx.x < K) L[threadIdx.x] = __ldcg(levels + threadIdx.x);
+    __syncthreads();
+    // level m + 1 from quads (one a thread: a tile has at most 16 x 16)
+    int cur = cur0, row0 = 0;
+    float4 *bufA = smem4, *bufB = smem4 + (size_t)cur * cur * C4;
+    static_assert(kNT >= 16 * 16, "a thread a quad");
+    if (const int i = threadIdx.x; i < cur * cur) {
+        const int x = i & (cur - 1), y = i >> (nlev - 1);
+        const int gx = tx0 + 2 * x, gy = ty0 + 2 * y;
+        TexelChannels t[4];  // texels (0,0) (1,0) (0,1) (1,1)
+        if (FROM_TEXELS) {
+#pragma unroll
+            for (int h = 0; h < 4; ++h) t[h] = texel_channels(tex[h], scale, K, L, log_w != 0);
+        }
+        // Whole 32-byte sectors at a time: the colours of two texels, the weights
+        // of one (two at K <= 4); every texel with an even column is 32-byte aligned.
+        const float3 w = rw[y];
+        float4 v[4], u[4];  // a slot of the four texels, and the next
+        auto slot = [&](int c, float4 (&o)[4]) {
+#pragma unroll
+            for (int h = 0; h < 4; ++h)
+                o[h] = FROM_TEXELS
+                           ? t[h].slot(c)
+                           : __ldcg(pyr + pyr_slot<C4>(rgb4[m], w4[m], gx + (h & 1), gy + (h >> 1), Ws, c));
+        };
+        auto put = [&](int r, int h, int c, const float4 &a, const float4 &b) {
+            if (FROM_TEXELS) st8(pyr + pyr_slot<C4>(rgb4[0], w4[0], gx + h, gy + r, Ws, c), a, b);
+        };
+        auto up = [&](int c) { return pyr + pyr_slot<C4>(rgb4[m + 1], w4[m + 1], gx >> 1, gy >> 1, Ws >> 1, c); };
+        slot(0, v);
+        put(0, 0, 0, v[0], v[1]);
+        put(1, 0, 0, v[2], v[3]);
+        *up(0) = bufA[i * C4] = mean4(v[0], v[1], v[2], v[3], w);
+        if constexpr (C4 == 2) {
+            slot(1, v);
+            put(0, 0, 1, v[0], v[1]);
+            put(1, 0, 1, v[2], v[3]);
+            *up(1) = bufA[i * C4 + 1] = mean4(v[0], v[1], v[2], v[3], w);
         } else {
 #pragma unroll
-            for (int c = 0; c < C4; ++c)
-                v[c] = __ldcg(pyr + pyr_slot<C4>(rgb4[m], w4[m], tx0 + lx, ty0 + ly, Ws, c));
+            for (int c = 1; c < C4; c += 2) {
+                slot(c, v);
+                slot(c + 1, u);
+#pragma unroll
+                for (int h = 0; h < 4; ++h) put(h >> 1, h & 1, c, v[h], u[h]);
+                const float4 r0 = mean4(v[0], v[1], v[2], v[3], w), r1 = mean4(u[0], u[1], u[2], u[3], w);
+                bufA[i * C4 + c] = r0;
+                bufA[i * C4 + c + 1] = r1;
+                st8(up(c), r0, r1);
+            }
         }
     }
     __syncthreads();
-    int cur = T;
-    for (int l = 1; l <= nlev; ++l) {
+    for (int l = 2; l <= nlev; ++l) {
         const int nxt = cur / 2, lg = nlev - l;  // nxt = 2^lg
-        const int Hp = Hs >> (l - 1), Wd = Ws >> l;  // parent height, level width
-        const float half = 0.5f * kPi / (float)Hp;
+        row0 += cur;
         const int X0 = tx0 >> l, Y0 = ty0 >> l;
-        if (threadIdx.x < nxt) {
-            const int Y = Y0 + threadIdx.x;
-            const float w0 = sinf((2.f * Y + 0.5f) * (kPi / (float)Hp)) * sinf(half);
-            const float w1 = sinf((2.f * Y + 1.5f) * (kPi / (float)Hp)) * sinf(half);
-            rw[threadIdx.x] = make_float4(w0, w1, 1.f / (2.f * (w0 + w1)), 0.f);
-        }
-        __syncthreads();
         for (int i = threadIdx.x; i < nxt * nxt * C4; i += kNT) {
             const int c = i % C4, t = i / C4;  // C4 is a constant: no division
             const int x = t & (nxt - 1), y = t >> lg;
-            const float4 wr = rw[y];
-            const float w0 = wr.x, w1 = wr.y, inv = wr.z;
-            const float4 a0 = bufA[((2 * y) * cur + 2 * x) * C4 + c];
-            const float4 a1 = bufA[((2 * y) * cur + 2 * x + 1) * C4 + c];
-            const float4 b0 = bufA[((2 * y + 1) * cur + 2 * x) * C4 + c];
-            const float4 b1 = bufA[((2 * y + 1) * cur + 2 * x + 1) * C4 + c];
-            float4 r;
-            r.x = (w0 * (a0.x + a1.x) + w1 * (b0.x + b1.x)) * inv;
-            r.y = (w0 * (a0.y + a1.y) + w1 * (b0.y + b1.y)) * inv;
-            r.z = (w0 * (a0.z + a1.z) + w1 * (b0.z + b1.z)) * inv;
-            r.w = (w0 * (a0.w + a1.w) + w1 * (b0.w + b1.w)) * inv;
+            const float4 *p = bufA + ((2 * y) * cur + 2 * x) * C4 + c;
+            const float4 r = mean4(p[0], p[C4], p[cur * C4], p[(cur + 1) * C4], rw[row0 + y]);
             bufB[t * C4 + c] = r;
-            pyr[pyr_slot<C4>(rgb4[m + l], w4[m + l], X0 + x, Y0 + y, Wd, c)] = r;
+            pyr[pyr_slot<C4>(rgb4[m + l], w4[m + l], X0 + x, Y0 + y, Ws >> l, c)] = r;
         }
         __syncthreads();  // (also: every store of the level issued before the block is counted as done)
         float4 *tmp = bufA;
@@ -244,25 +355,29 @@ __global__ void __launch_bounds__(kNT) k_pyramid(const void *__restrict__ texels
     if (!last) return;
     __threadfence();
     int Wc = Ws >> nlev, Hc = Hs >> nlev;  // level m + nlev, the parent of the first tail level
+    bufA = smem4;
+    bufB = smem4 + (size_t)C4 * (kPyrTailTexels / 4);
     for (int l = m + nlev + 1; l <= tail_to; ++l) {
         const int Wd = Wc / 2, Hd = Hc / 2;
-        const float half = 0.5f * kPi / (float)Hc;
+        const bool first = l == m + nlev + 1;
+        float4 *dst = ((l - m - nlev) & 1) ? bufA : bufB;
+        const float4 *src = ((l - m - nlev) & 1) ? bufB : bufA;
         for (int i = threadIdx.x; i < Wd * Hd * C4; i += kNT) {
             const int c = i % C4, t = i / C4;
-            const int x = t % Wd, Y = t / Wd;
-            const float w0 = sinf((2.f * Y + 0.5f) * (kPi / (float)Hc)) * sinf(half);
-            const float w1 = sinf((2.f * Y + 1.5f) * (kPi / (float)Hc)) * sinf(half);
-            const size_t r4 = rgb4[l - 1], ww4 = w4[l - 1];
-            const float4 a0 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x, 2 * Y, Wc, c));
-            const float4 a1 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x + 1, 2 * Y, Wc, c));
-            const float4 b0 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x, 2 * Y + 1, Wc, c));
-            const float4 b1 = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x + 1, 2 * Y + 1, Wc, c));
-            const float inv = 1.f / (2.f * (w0 + w1));
-            float4 r;
-            r.x = (w0 * (a0.x + a1.x) + w1 * (b0.x + b1.x)) * inv;
-            r.y = (w0 * (a0.y + a1.y) + w1 * (b0.y + b1.y)) * inv;
-            r.z = (w0 * (a0.z + a1.z) + w1 * (b0.z + b1.z)) * inv;
-            r.w = (w0 * (a0.w + a1.w) + w1 * (b0.w + b1.w)) * inv;
+            const int x = t & (Wd - 1), Y = t / Wd;
+            const float3 w = row_weights(Y, Hc);
+            float4 ch[4];
+            if (first) {
+                const size_t r4 = rgb4[l - 1], ww4 = w4[l - 1];
+#pragma unroll
+                for (int h = 0; h < 4; ++h)
+                    ch[h] = __ldcg(pyr + pyr_slot<C4>(r4, ww4, 2 * x + (h & 1), 2 * Y + (h >> 1), Wc, c));
+            } else {
+                const float4 *p = src + ((2 * Y) * Wc + 2 * x) * C4 + c;
+                ch[0] = p[0]; ch[1] = p[C4]; ch[2] = p[Wc * C4]; ch[3] = p[(Wc + 1) * C4];
+            }
+            const float4 r = mean4(ch[0], ch[1], ch[2], ch[3], w);
+            dst[t * C4 + c] = r;
             pyr[pyr_slot<C4>(rgb4[l], w4[l], x, Y, Wd, c)] = r;
         }
         __syncthreads();  // level l complete before it is read
@@ -271,10 +386,6 @@ __global__ void __launch_bounds__(kNT) k_pyramid(const void *__restrict__ texels
     }
     if (threadIdx.x == 0) *done = 0u;
 }
-
-// Upper pyramid levels whose base holds at most this many texels are built
-// by the last block of the launch that writes the base.
-constexpr long kPyrTailTexels = 2048;
 
 // Step 5a: filter sample table (Hammersley points mapped through the GGX
 // distribution of microfacet normals weighted by cos theta_h):
@@ -339,107 +450,13 @@ struct FilterLevels {
 
 constexpr int kFilterSplit = 2;  // threads per output texel (samples strided over them)
 
+// Filtered texel `at` from the sums over its nv samples: the record in the
+// stored format and the weights-only copy.
 template <int C4>
-__global__ void __launch_bounds__(128) k_filter(const float4 *__restrict__ pyr, const size_t *__restrict__ rgb4,
-                                                  const size_t *__restrict__ w4,
-                                                  int W, int H, int M, const float4 *__restrict__ table,
-                                                  const int *__restrict__ nvalid, int S, const FilterLevels fl,
-                                                  float4 *__restrict__ out, float4 *__restrict__ outw, int wfmt,
-                                                  int rec4, int K) {
-    extern __shared__ float4 tab[];
-    int r = 0;
-    while (r + 1 < fl.nlev && (int)blockIdx.x >= fl.blk[r + 1]) ++r;
-    const int Wo = fl.width[r], Ho = Wo / 2;
-    const int nv = nvalid[r];
-    for (int k = threadIdx.x; k < nv; k += blockDim.x) tab[k] = table[(size_t)r * S + k];
-    __syncthreads();
-    const int g = threadIdx.x % kFilterSplit;
-    const int t = ((int)blockIdx.x - fl.blk[r]) * (blockDim.x / kFilterSplit) + threadIdx.x / kFilterSplit;
-    const bool active = t < Wo * Ho;
-    const int tt = active ? t : 0;
-    const int x = tt % Wo, y = tt / Wo;
-    const float th = kPi * ((float)y + 0.5f) / (float)Ho;
-    const float ph = kTwoPi * ((float)x + 0.5f) / (float)Wo;
-    float st, ct, sp, cp;
-    sincosf(th, &st, &ct);
-    sincosf(ph, &sp, &cp);
-    const float rx = st * cp, ry = ct, rz = st * sp;
-    const float e1x = ct * cp, e1y = -st, e1z = ct * sp;
-    const float e2x = -sp, e2z = cp;
-    // colour and weights accumulated apart (the pyramid's split storage);
-    // every channel goes through the same multiply-adds as in the record layout
+__device__ __forceinline__ void store_filtered(const float4 &accr, const float4 *accw, int nv, size_t at,
+                                               float4 *__restrict__ out, float4 *__restrict__ outw, int wfmt, int rec4,
+                                               int K) {
     constexpr int KW4 = C4 - 1;
-    float4 accr = make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 accw[KW4];
-#pragma unroll
-    for (int c = 0; c < KW4; ++c) accw[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int k = g; k < nv; k += kFilterSplit) {
-        const float4 smp = tab[k];
-        const float dx = smp.x * e1x + smp.y * e2x + smp.z * rx;
-        const float dy = smp.x * e1y + smp.z * ry;
-        const float dz = smp.x * e1z + smp.y * e2z + smp.z * rz;
-        const float lod = smp.w;
-        const int m0 = (int)floorf(lod);
-        const float f = lod - (float)m0;
-        const int m1 = min(m0 + 1, M - 1);
-        const float th_i = acosf(fminf(fmaxf(dy, -1.f), 1.f));
-        float ph_i = atan2f(dz, dx);
-        if (ph_i < 0.f) ph_i += kTwoPi;
-#pragma unroll
-        for (int lv = 0; lv < 2; ++lv) {
-            const int m = lv ? m1 : m0;
-            const float wl = lv ? f : 1.f - f;
-            const int Wm = W >> m, Hm = H >> m;
-            const float xx = ph_i * (kInvTwoPi * (float)Wm) - 0.5f;
-            const float yy = th_i * (kInvPi * (float)Hm) - 0.5f;
-            const Taps tp = equirect_taps(xx, yy, Wm, Hm);
-            const float4 *prgb = pyr + rgb4[m], *pw = pyr + w4[m];
-            const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
-            // pyr_column of the weights
-            const int s0 = KW4 >= 2 && (tp.i00 & Wm) ? 2 : 0, s1 = KW4 >= 2 && (tp.i10 & Wm) ? 2 : 0;
-            const int widx[4] = {tp.i00 ^ s0, tp.i01 ^ s0, tp.i10 ^ s1, tp.i11 ^ s1};
-            float4 tr[4], tw[4][KW4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                tr[j] = __ldg(prgb + idx[j]);
-                if constexpr (KW4 == 2) {
-                    ldg8(pw + (size_t)widx[j] * 2, tw[j][0], tw[j][1]);  // 32-byte aligned (even level offsets)
-                } else {
-#pragma unroll
-                    for (int c = 0; c < KW4; ++c) tw[j][c] = __ldg(pw + (size_t)widx[j] * KW4 + c);
-                }
-            }
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            v = fma4(tp.w00, tr[0], v);
-            v = fma4(tp.w01, tr[1], v);
-            v = fma4(tp.w10, tr[2], v);
-            v = fma4(tp.w11, tr[3], v);
-            accr = fma4(wl, v, accr);
-#pragma unroll
-            for (int c = 0; c < KW4; ++c) {
-                float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                u = fma4(tp.w00, tw[0][c], u);
-                u = fma4(tp.w01, tw[1][c], u);
-                u = fma4(tp.w10, tw[2][c], u);
-                u = fma4(tp.w11, tw[3][c], u);
-                accw[c] = fma4(wl, u, accw[c]);
-            }
-        }
-    }
-    // sum the partial means of the kFilterSplit adjacent lanes of a texel
-#pragma unroll
-    for (int o = 1; o < kFilterSplit; o <<= 1) {
-        accr.x += __shfl_xor_sync(0xffffffffu, accr.x, o);
-        accr.y += __shfl_xor_sync(0xffffffffu, accr.y, o);
-        accr.z += __shfl_xor_sync(0xffffffffu, accr.z, o);
-#pragma unroll
-        for (int c = 0; c < KW4; ++c) {
-            accw[c].x += __shfl_xor_sync(0xffffffffu, accw[c].x, o);
-            accw[c].y += __shfl_xor_sync(0xffffffffu, accw[c].y, o);
-            accw[c].z += __shfl_xor_sync(0xffffffffu, accw[c].z, o);
-            accw[c].w += __shfl_xor_sync(0xffffffffu, accw[c].w, o);
-        }
-    }
     // back to the record layout (R, G, B, W_1 .. W_K, zero padding)
     float4 acc[C4];
     {
@@ -453,12 +470,11 @@ __global__ void __launch_bounds__(128) k_filter(const float4 *__restrict__ pyr, 
 #pragma unroll
         for (int c = 0; c < C4; ++c) acc[c] = make_float4(ch[4 * c], ch[4 * c + 1], ch[4 * c + 2], ch[4 * c + 3]);
     }
-    if (!active || g != 0) return;
     const float inv = nv > 0 ? 1.f / (float)nv : 0.f;
     const int kw4 = (K + 3) / 4;
-    float4 *ow = outw + ((size_t)fl.off[r] + t) * kw4;
+    float4 *ow = outw + at * kw4;
     if (wfmt == GLINT_WFMT_F32) {
-        float4 *o = out + ((size_t)fl.off[r] + t) * C4;
+        float4 *o = out + at * C4;
         float ch[C4 * 4 + 4];
 #pragma unroll
         for (int c = 0; c < C4; ++c) {
@@ -482,7 +498,7 @@ __global__ void __launch_bounds__(128) k_filter(const float4 *__restrict__ pyr, 
         ch[4 * c] = acc[c].x * inv; ch[4 * c + 1] = acc[c].y * inv;
         ch[4 * c + 2] = acc[c].z * inv; ch[4 * c + 3] = acc[c].w * inv;
     }
-    float4 *o = out + ((size_t)fl.off[r] + t) * rec4;
+    float4 *o = out + at * rec4;
     o[0] = make_float4(ch[0], ch[1], ch[2], 0.f);
     uint32_t words[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
     float dec[C4 * 4];  // the weights as the stored codes decode
@@ -511,26 +527,245 @@ __global__ void __launch_bounds__(128) k_filter(const float4 *__restrict__ pyr, 
     for (int i = 0; i < rec4 - 1; ++i) q[i] = make_uint4(words[4 * i], words[4 * i + 1], words[4 * i + 2], words[4 * i + 3]);
 }
 
+// One sample's trilinear look-up at direction (dx, dy, dz): the bilinear values
+// of the two levels bracketing lod, colour and weights apart (the pyramid's
+// split storage); sink(wl, v, u) takes them in order.  A level that weighs
+// nothing (lod at either end of the pyramid) is not read.
+template <int C4, class Sink>
+__device__ __forceinline__ void filter_sample(const float4 *__restrict__ pyr, const size_t *__restrict__ rgb4,
+                                              const size_t *__restrict__ w4, int W, int H, int M, float dx, float dy,
+                                              float dz, float lod, Sink &&sink) {
+    constexpr int KW4 = C4 - 1;
+    const int m0 = (int)floorf(lod);
+    const float f = lod - (float)m0;
+    const int m1 = min(m0 + 1, M - 1);
+    const float th_i = acosf(fminf(fmaxf(dy, -1.f), 1.f));
+    float ph_i = atan2f(dz, dx);
+    if (ph_i < 0.f) ph_i += kTwoPi;
+#pragma unroll
+    for (int lv = 0; lv < 2; ++lv) {
+        if (lv == 1 && f == 0.f) break;
+        const int m = lv ? m1 : m0;
+        const float wl = lv ? f : 1.f - f;
+        const int Wm = W >> m, Hm = H >> m;
+        const float xx = ph_i * (kInvTwoPi * (float)Wm) - 0.5f;
+        const float yy = th_i * (kInvPi * (float)Hm) - 0.5f;
+        const Taps tp = equirect_taps(xx, yy, Wm, Hm);
+        const float4 *prgb = pyr + rgb4[m], *pw = pyr + w4[m];
+        const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
+        // pyr_column of the weights
+        const int s0 = KW4 >= 2 && (tp.i00 & Wm) ? 2 : 0, s1 = KW4 >= 2 && (tp.i10 & Wm) ? 2 : 0;
+        const int widx[4] = {tp.i00 ^ s0, tp.i01 ^ s0, tp.i10 ^ s1, tp.i11 ^ s1};
+        float4 tr[4], tw[4][KW4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            tr[j] = __ldg(prgb + idx[j]);
+            ldg_texel<KW4>(pw + (size_t)widx[j] * KW4, tw[j]);
+        }
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u[KW4];
+        v = fma4(tp.w00, tr[0], v);
+        v = fma4(tp.w01, tr[1], v);
+        v = fma4(tp.w10, tr[2], v);
+        v = fma4(tp.w11, tr[3], v);
+#pragma unroll
+        for (int c = 0; c < KW4; ++c) {
+            u[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+            u[c] = fma4(tp.w00, tw[0][c], u[c]);
+            u[c] = fma4(tp.w01, tw[1][c], u[c]);
+            u[c] = fma4(tp.w10, tw[2][c], u[c]);
+            u[c] = fma4(tp.w11, tw[3][c], u[c]);
+        }
+        sink(lv, wl, v, u);
+    }
+}
+
+// Frame of an output texel: its direction r and e1 = d r / d theta, e2 =
+// d r / d phi / sin theta (e2.y = 0).
+struct FilterFrame {
+    float rx, ry, rz, e1x, e1y, e1z, e2x, e2z;
+    __device__ __forceinline__ FilterFrame(int x, int y, int Wo, int Ho) {
+        const float th = kPi * ((float)y + 0.5f) / (float)Ho;
+        const float ph = kTwoPi * ((float)x + 0.5f) / (float)Wo;
+        float st, ct, sp, cp;
+        sincosf(th, &st, &ct);
+        sincosf(ph, &sp, &cp);
+        rx = st * cp; ry = ct; rz = st * sp;
+        e1x = ct * cp; e1y = -st; e1z = ct * sp;
+        e2x = -sp; e2z = cp;
+    }
+};
+
+template <int C4>
+__global__ void __launch_bounds__(128) k_filter(const float4 *__restrict__ pyr, const size_t *__restrict__ rgb4,
+                                                  const size_t *__restrict__ w4,
+                                                  int W, int H, int M, const float4 *__restrict__ table,
+                                                  const int *__restrict__ nvalid, int S, const FilterLevels fl,
+                                                  float4 *__restrict__ out, float4 *__restrict__ outw, int wfmt,
+                                                  int rec4, int K) {
+    extern __shared__ float4 tab[];
+    int r = 0;
+    while (r + 1 < fl.nlev && (int)blockIdx.x >= fl.blk[r + 1]) ++r;
+    const int Wo = fl.width[r], Ho = Wo / 2;
+    const int nv = nvalid[r];  // (the table is the environment's own since its creation)
+    for (int k = threadIdx.x; k < nv; k += blockDim.x) tab[k] = table[(size_t)r * S + k];
+    __syncthreads();
+    const int g = threadIdx.x % kFilterSplit;
+    const int t = ((int)blockIdx.x - fl.blk[r]) * (blockDim.x / kFilterSplit) + threadIdx.x / kFilterSplit;
+    const bool active = t < Wo * Ho;
+    const int tt = active ? t : 0;
+    const int x = tt % Wo, y = tt / Wo;
+    const FilterFrame fr(x, y, Wo, Ho);
+    pdl_wait_then_release();
+    // colour and weights accumulated apart (the pyramid's split storage);
+    // every channel goes through the same multiply-adds as in the record layout
+    constexpr int KW4 = C4 - 1;
+    float4 accr = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 accw[KW4];
+#pragma unroll
+    for (int c = 0; c < KW4; ++c) accw[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int k = g; k < nv; k += kFilterSplit) {
+        const float4 smp = tab[k];
+        const float dx = smp.x * fr.e1x + smp.y * fr.e2x + smp.z * fr.rx;
+        const float dy = smp.x * fr.e1y + smp.z * fr.ry;
+        const float dz = smp.x * fr.e1z + smp.y * fr.e2z + smp.z * fr.rz;
+        filter_sample<C4>(pyr, rgb4, w4, W, H, M, dx, dy, dz, smp.w,
+                          [&](int, float wl, const float4 &v, const float4(&u)[KW4]) {
+                              accr = fma4(wl, v, accr);
+#pragma unroll
+                              for (int c = 0; c < KW4; ++c) accw[c] = fma4(wl, u[c], accw[c]);
+                          });
+    }
+    // sum the partial means of the kFilterSplit adjacent lanes of a texel
+#pragma unroll
+    for (int o = 1; o < kFilterSplit; o <<= 1) {
+        accr.x += __shfl_xor_sync(0xffffffffu, accr.x, o);
+        accr.y += __shfl_xor_sync(0xffffffffu, accr.y, o);
+        accr.z += __shfl_xor_sync(0xffffffffu, accr.z, o);
+#pragma unroll
+        for (int c = 0; c < KW4; ++c) {
+            accw[c].x += __shfl_xor_sync(0xffffffffu, accw[c].x, o);
+            accw[c].y += __shfl_xor_sync(0xffffffffu, accw[c].y, o);
+            accw[c].z += __shfl_xor_sync(0xffffffffu, accw[c].z, o);
+            accw[c].w += __shfl_xor_sync(0xffffffffu, accw[c].w, o);
+        }
+    }
+    if (!active || g != 0) return;
+    store_filtered<C4>(accr, accw, nv, (size_t)fl.off[r] + t, out, outw, wfmt, rec4, K);
+}
+
+// The same filtered maps where they are too few for k_filter to fill the chip
+// (latency-bound: a thread there takes 32 of 64 samples one after the other).  A
+// thread takes one sample of one texel, kFilterSamples samples of a texel at a
+// time; their values go to shared memory, and a thread for each channel and
+// parity of the sample adds them up in the order k_filter does, so the sums are
+// the same.  Twice the instructions a sample, so up to 64 texels an SM only (map
+// update and a 16 x 16 frame, us, k_filter / this; 400 texels, K = 4, 8, 16: 39 /
+// 27, 52 / 32, 90 / 43; 7456, K = 4, 8: 65 / 55, 91 / 71; 19808: 59 / 77, 79 / 95).
+constexpr int kFilterSmall = 64;
+constexpr int kFilterTexels = 4, kFilterSamples = 64;  // per block: 256 threads
+
+template <int C4>
+__global__ void __launch_bounds__(kFilterTexels * kFilterSamples) k_filter_small(
+    const float4 *__restrict__ pyr, const size_t *__restrict__ rgb4, const size_t *__restrict__ w4, int W, int H, int M,
+    const float4 *__restrict__ table, const int *__restrict__ nvalid, int S, const FilterLevels fl,
+    float4 *__restrict__ out, float4 *__restrict__ outw, int wfmt, int rec4, int K) {
+    constexpr int KW4 = C4 - 1, Cpad = 4 * C4;
+    constexpr int kStride = 2 * C4 + 1;  // float4 per sample: both levels, odd (no bank conflicts)
+    extern __shared__ float4 vals[];     // [texel][sample][kStride]
+    __shared__ float wts[kFilterSamples][2];
+    __shared__ float sums[kFilterTexels][2][Cpad];
+    int r = 0;
+    while (r + 1 < fl.nlev && (int)blockIdx.x >= fl.blk[r + 1]) ++r;
+    const int Wo = fl.width[r], Ho = Wo / 2;
+    const int nv = nvalid[r];
+    const int t0 = ((int)blockIdx.x - fl.blk[r]) * kFilterTexels;
+    const int tx = threadIdx.x / kFilterSamples, kk = threadIdx.x % kFilterSamples;
+    const int t = min(t0 + tx, Wo * Ho - 1);
+    const FilterFrame fr(t % Wo, t / Wo, Wo, Ho);
+    // the adder of channel ch, parity g, texel at
+    const int ch = threadIdx.x % Cpad, g = threadIdx.x / Cpad % 2, at = threadIdx.x / (2 * Cpad);
+    pdl_wait_then_release();
+    float acc = 0.f;
+    for (int k0 = 0; k0 < nv; k0 += kFilterSamples) {
+        const int k = k0 + kk;
+        if (k < nv) {
+            const float4 smp = __ldg(table + (size_t)r * S + k);
+            const float dx = smp.x * fr.e1x + smp.y * fr.e2x + smp.z * fr.rx;
+            const float dy = smp.x * fr.e1y + smp.z * fr.ry;
+            const float dz = smp.x * fr.e1z + smp.y * fr.e2z + smp.z * fr.rz;
+            float4 *o = vals + threadIdx.x * kStride;
+            if (tx == 0) wts[kk][1] = 0.f;
+            filter_sample<C4>(pyr, rgb4, w4, W, H, M, dx, dy, dz, smp.w,
+                              [&](int lv, float wl, const float4 &v, const float4(&u)[KW4]) {
+                                  if (tx == 0) wts[kk][lv] = wl;
+                                  o[lv * C4] = v;
+#pragma unroll
+                                  for (int c = 0; c < KW4; ++c) o[lv * C4 + 1 + c] = u[c];
+                              });
+        }
+        __syncthreads();
+        if (at < kFilterTexels) {
+            const float *v = reinterpret_cast<const float *>(vals + at * kFilterSamples * kStride) + ch;
+            const int n = min(kFilterSamples, nv - k0);
+#pragma unroll 4
+            for (int i = g; i < n; i += kFilterSplit) {  // (k0 is even)
+                acc = fmaf(wts[i][0], v[i * 4 * kStride], acc);
+                if (wts[i][1] != 0.f) acc = fmaf(wts[i][1], v[i * 4 * kStride + Cpad], acc);
+            }
+        }
+        __syncthreads();
+    }
+    if (at < kFilterTexels) sums[at][g][ch] = acc;
+    __syncthreads();
+    if (threadIdx.x < kFilterTexels && t0 + (int)threadIdx.x < Wo * Ho) {
+        const float *s0 = sums[threadIdx.x][0], *s1 = sums[threadIdx.x][1];
+        float4 a[C4];
+#pragma unroll
+        for (int c = 0; c < C4; ++c)
+            a[c] = make_float4(s0[4 * c] + s1[4 * c], s0[4 * c + 1] + s1[4 * c + 1], s0[4 * c + 2] + s1[4 * c + 2],
+                               s0[4 * c + 3] + s1[4 * c + 3]);
+        store_filtered<C4>(a[0], a + 1, nv, (size_t)fl.off[r] + t0 + threadIdx.x, out, outw, wfmt, rec4, K);
+    }
+}
+static_assert(kFilterSplit == 2 && kFilterTexels * 2 * 20 <= kFilterTexels * kFilterSamples, "an adder a channel and parity");
+
 }  // namespace
 
 template <int C4>
-cudaError_t launch_pyramid(bool first, unsigned blocks, size_t smem, cudaStream_t s, const void *texels,
-                           const glint_env_desc &d, float scale, glint_env *env, int m, int Ws, int Hs, int T, int nlev,
-                           int tail_to) {
-    if (first) {
-        cudaFuncSetAttribute(k_pyramid<true, C4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pyramid<true, C4><<<blocks, kNT, smem, s>>>(texels, d.format, scale, d.K, env->levels,
-                                                       reinterpret_cast<float4 *>(env->pyr), env->pyr_rgb4_dev,
-                                                       env->pyr_w4_dev, 0, Ws, Hs, T, nlev, d.weight_space, tail_to,
-                                                       env->done + 1);
-    } else {
-        cudaFuncSetAttribute(k_pyramid<false, C4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_pyramid<false, C4><<<blocks, kNT, smem, s>>>(nullptr, d.format, scale, d.K, env->levels,
-                                                        reinterpret_cast<float4 *>(env->pyr), env->pyr_rgb4_dev,
-                                                        env->pyr_w4_dev, m, Ws, Hs, T, nlev, 0, tail_to,
-                                                        env->done + 1);
+cudaError_t launch_pyramid(bool first, unsigned blocks, cudaStream_t s, const void *texels, const glint_env_desc &d,
+                           float scale, glint_env *env, int m, int Ws, int Hs, int T, int nlev, int tail_to, bool wide) {
+    const size_t smem = pyramid_smem<C4>();
+    auto *pyr = reinterpret_cast<float4 *>(env->pyr);
+    const float *levels = env->levels;
+    const size_t *rgb4 = env->pyr_rgb4_dev, *w4 = env->pyr_w4_dev;
+    auto kernel = first ? k_pyramid<true, C4> : k_pyramid<false, C4>;
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
     }
-    return cudaGetLastError();
+    return launch_pdl(true, kernel, blocks, kNT, smem, s, first ? texels : nullptr, d.format, scale, d.K, levels, pyr,
+                      rgb4, w4, m, Ws, Hs, T, nlev, d.weight_space, tail_to, env->done + 1, wide);
+}
+
+template <int C4>
+cudaError_t launch_filter(glint_env *env, const FilterLevels &fl, int blk, bool small, cudaStream_t s) {
+    const glint_env_desc &d = env->d;
+    const float4 *pyr4 = reinterpret_cast<const float4 *>(env->pyr), *table = env->table;
+    float4 *out4 = reinterpret_cast<float4 *>(env->filt);
+    const size_t *rgb4 = env->pyr_rgb4_dev, *w4 = env->pyr_w4_dev;
+    const int *nvalid = env->nvalid;
+    auto kernel = small ? k_filter_small<C4> : k_filter<C4>;
+    const unsigned threads = small ? kFilterTexels * kFilterSamples : 128;
+    const size_t smem = sizeof(float4) * (small ? (size_t)kFilterTexels * kFilterSamples * (2 * C4 + 1) : (size_t)d.samples);
+    if (smem > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    // Not early for k_filter: it is one wave of blocks bound by the L1s, and blocks
+    // placed while the pyramid still runs crowd the SMs that are free first (1024 x
+    // 512 map: K = 8 the update 30 us longer, K = 16 240 us).
+    return launch_pdl(small, kernel, blk, threads, smem, s, pyr4, rgb4, w4, d.width, d.height, env->M, table, nvalid,
+                      d.samples, fl, out4, env->filtw, d.weight_format, env->frec4, d.K);
 }
 
 // Pyramid level offsets (float4 units) are in a small device array that
@@ -540,10 +775,11 @@ cudaError_t glint_launch_env(glint_env *env, const void *texels, cudaStream_t s,
     const long n = (long)d.width * d.height;
     const float scale = ldexpf(1.f, d.scale_log2);
     const int C4 = env->Cpad / 4;
-    (void)n;
     int nl = 0;
-    k_minmax<<<env->nblk_minmax, kNT, 0, s>>>(texels, d.format, n, scale, env->partial, env->done, d.K, d.ell,
-                                                env->levels);
+    const bool wide = ((uintptr_t)texels & 15u) == 0;
+    const long per_block = 2L * kNT * kMinMaxPairs;
+    const int nblk = wide ? (int)std::min<long>(env->nblk_minmax, (n + per_block - 1) / per_block) : env->nblk_minmax;
+    k_minmax<<<nblk, kNT, 0, s>>>(texels, d.format, n, scale, env->partial, env->done, d.K, d.ell, env->levels, wide);
     ++nl;
     {
         // level 0 and the next log2 T levels from the texels (T = 32), then
@@ -559,13 +795,12 @@ cudaError_t glint_launch_env(glint_env *env, const void *texels, cudaStream_t s,
             while ((1 << nlev) < T) ++nlev;
             const bool tail = m + nlev < env->M - 1 && (long)(Ws >> nlev) * (Hs >> nlev) <= kPyrTailTexels;
             const int tail_to = tail ? env->M - 1 : -1;
-            const size_t smem = sizeof(float) * env->Cpad * ((size_t)T * T + (size_t)(T / 2) * (T / 2));
             const unsigned blocks = (unsigned)((Ws / T) * (Hs / T));
             cudaError_t e = cudaSuccess;
             switch (C4) {
-            case 2: e = launch_pyramid<2>(first, blocks, smem, s, texels, d, scale, env, m, Ws, Hs, T, nlev, tail_to); break;
-            case 3: e = launch_pyramid<3>(first, blocks, smem, s, texels, d, scale, env, m, Ws, Hs, T, nlev, tail_to); break;
-            case 5: e = launch_pyramid<5>(first, blocks, smem, s, texels, d, scale, env, m, Ws, Hs, T, nlev, tail_to); break;
+            case 2: e = launch_pyramid<2>(first, blocks, s, texels, d, scale, env, m, Ws, Hs, T, nlev, tail_to, wide); break;
+            case 3: e = launch_pyramid<3>(first, blocks, s, texels, d, scale, env, m, Ws, Hs, T, nlev, tail_to, wide); break;
+            case 5: e = launch_pyramid<5>(first, blocks, s, texels, d, scale, env, m, Ws, Hs, T, nlev, tail_to, wide); break;
             default: return cudaErrorInvalidValue;
             }
             if (e != cudaSuccess) return e;
@@ -580,34 +815,25 @@ cudaError_t glint_launch_env(glint_env *env, const void *texels, cudaStream_t s,
     {
         FilterLevels fl{};
         fl.nlev = d.levels;
+        // below kFilterSmall texels an SM the samples of a texel run side by side
+        const bool small = env->foff[d.levels] < (long long)kFilterSmall * env->ctx->num_sms;
+        const int per_block = small ? kFilterTexels : 128 / kFilterSplit;
         int blk = 0;
         for (int r = 0; r < d.levels; ++r) {
             fl.width[r] = env->fw[r];
             fl.off[r] = env->foff[r];
             fl.blk[r] = blk;
-            const int per_block = 128 / kFilterSplit;
             blk += (int)((env->fw[r] * (env->fw[r] / 2) + per_block - 1) / per_block);
         }
         fl.blk[d.levels] = blk;
-        const size_t smem = sizeof(float4) * (size_t)d.samples;
-        const float4 *pyr4 = reinterpret_cast<const float4 *>(env->pyr);
-        float4 *out4 = reinterpret_cast<float4 *>(env->filt);
+        cudaError_t e = cudaSuccess;
         switch (C4) {
-        case 2:
-            k_filter<2><<<blk, 128, smem, s>>>(pyr4, env->pyr_rgb4_dev, env->pyr_w4_dev, d.width, d.height, env->M, env->table, env->nvalid,
-                                               d.samples, fl, out4, env->filtw, d.weight_format, env->frec4, d.K);
-            break;
-        case 3:
-            k_filter<3><<<blk, 128, smem, s>>>(pyr4, env->pyr_rgb4_dev, env->pyr_w4_dev, d.width, d.height, env->M, env->table, env->nvalid,
-                                               d.samples, fl, out4, env->filtw, d.weight_format, env->frec4, d.K);
-            break;
-        case 5:
-            k_filter<5><<<blk, 128, smem, s>>>(pyr4, env->pyr_rgb4_dev, env->pyr_w4_dev, d.width, d.height, env->M, env->table, env->nvalid,
-                                               d.samples, fl, out4, env->filtw, d.weight_format, env->frec4, d.K);
-            break;
-        default:
-            return cudaErrorInvalidValue;
+        case 2: e = launch_filter<2>(env, fl, blk, small, s); break;
+        case 3: e = launch_filter<3>(env, fl, blk, small, s); break;
+        case 5: e = launch_filter<5>(env, fl, blk, small, s); break;
+        default: return cudaErrorInvalidValue;
         }
+        if (e != cudaSuccess) return e;
         ++nl;
     }
     if (launches) *launches = nl;

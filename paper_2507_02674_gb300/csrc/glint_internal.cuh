@@ -235,10 +235,62 @@ __device__ __forceinline__ void ldg8(const float4 *p, float4 &lo, float4 &hi) {
         : "l"(p));
 }
 
+// A texel's KW4 float4 of weights; 32- and 64-byte texels (KW4 = 2, 4) in 256-bit
+// loads: they are 32-byte aligned in cudaMalloc'd buffers with even level
+// offsets.  (K = 16: 12 requests a look-up instead of 20.)
+template <int KW4>
+__device__ __forceinline__ void ldg_texel(const float4 *p, float4 (&t)[KW4]) {
+    if constexpr (KW4 == 1) {
+        t[0] = __ldg(p);
+    } else {
+        static_assert(KW4 % 2 == 0, "whole 32-byte pieces");
+#pragma unroll
+        for (int c = 0; c < KW4; c += 2) ldg8(p + c, t[c], t[c + 1]);
+    }
+}
+// and one 256-bit store
+__device__ __forceinline__ void st8(float4 *p, const float4 &lo, const float4 &hi) {
+    asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 :
+                 : "l"(p), "f"(lo.x), "f"(lo.y), "f"(lo.z), "f"(lo.w), "f"(hi.x), "f"(hi.y), "f"(hi.z), "f"(hi.w)
+                 : "memory");
+}
+
 __device__ __forceinline__ float4 fma4(float w, float4 a, float4 acc) {
     acc.x = fmaf(w, a.x, acc.x); acc.y = fmaf(w, a.y, acc.y);
     acc.z = fmaf(w, a.z, acc.z); acc.w = fmaf(w, a.w, acc.w);
     return acc;
+}
+
+// Programmatic dependent launch: a kernel launched with the attribute may have
+// its blocks resident while the stream's previous kernel still runs.
+// pdl_wait (before any read of memory that an earlier kernel may write, and
+// before any write) holds them until that kernel has completed and its writes
+// are visible; pdl_release lets the next kernel's blocks be scheduled once every
+// block of this one has started.  Without the launch attribute both do nothing.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_then_release() {
+    pdl_wait();
+    pdl_release();
+}
+
+// A launch whose blocks may start while the stream's previous kernel runs
+// (pdl), or an ordinary one.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                       Args... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
 }  // namespace glint

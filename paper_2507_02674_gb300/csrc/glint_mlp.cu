@@ -491,6 +491,7 @@ __global__ void __launch_bounds__(kFusedNT, 2) k_shade_mlp(ShadeArgs a, const __
                                                           const float *__restrict__ params) {
     extern __shared__ __align__(16) unsigned char fused_smem[];
     SmemFused &sm = *reinterpret_cast<SmemFused *>(fused_smem);
+    pdl_wait_then_release();
     load_weights<kFusedNT>(sm.w, wt, params);
     const long q = (long)blockIdx.x * kFusedNT + threadIdx.x;
     fused_tile<K, INTEGER, DEBUG>(a, sm, q, q < a.npix);
@@ -597,17 +598,6 @@ __device__ __forceinline__ void frag_b2(const __nv_bfloat16 *dz, int ld, int k0,
     // matrices: (k0.., n0), (k0 + 8.., n0), (k0.., n0 + 8), (k0 + 8.., n0 + 8)
     const int L = threadIdx.x & 31;
     ldsm_x4_trans(b, row_chunk_addr(dz, ld, k0 + (L & 7) + (((L >> 3) & 1) << 3), (n0 >> 3) + (L >> 4)));
-}
-
-// Programmatic dependent launch between the training kernels: a kernel's
-// blocks may become resident while the previous kernel of the stream still
-// runs; griddepcontrol.wait (first, before any global read or write) holds
-// them until that kernel has completed and its writes are visible, and
-// launch_dependents lets the next kernel's blocks be scheduled.  Without the
-// launch attribute both are no-ops.
-__device__ __forceinline__ void pdl_wait_then_release() {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <int NT>
@@ -1029,8 +1019,8 @@ cudaError_t launch_shade_mlp(const ShadeArgs &a, const glint_mlp *m, cudaStream_
                                          (int)smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((a.npix + kFusedNT - 1) / kFusedNT);
-    k_shade_mlp<K, INTEGER, DEBUG><<<grid, kFusedNT, smem, s>>>(a, m->wt, m->params);
-    return cudaGetLastError();
+    return launch_pdl(true, k_shade_mlp<K, INTEGER, DEBUG>, grid, kFusedNT, smem, s, a, (const __nv_bfloat16 *)m->wt,
+                      (const float *)m->params);
 }
 
 template <int K>
@@ -1091,27 +1081,6 @@ void glint_mlp_weights(const glint_mlp *g, const void **wt, const float **params
 
 int glint_mlp_k(const glint_mlp *g) { return g ? g->K : 0; }
 int glint_mlp_device(const glint_mlp *g) { return g ? g->device : -1; }
-
-namespace {
-// A launch whose blocks may start while the stream's previous kernel runs
-// (pdl: the kernel waits on it with pdl_wait_then_release), or an ordinary one.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                       cudaStream_t s, Args... args) {
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
-}
-
-}  // namespace
 
 extern "C" {
 

@@ -114,12 +114,7 @@ __device__ __forceinline__ void e2_probabilities(const ShadeArgs &a, long q, flo
             float4 tw[4][KW4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                if constexpr (KW4 == 2) {
-                    ldg8(levw + (size_t)idx[j] * 2, tw[j][0], tw[j][1]);  // 32-byte aligned (even level offsets)
-                } else {
-#pragma unroll
-                    for (int c = 0; c < KW4; ++c) tw[j][c] = __ldg(levw + (size_t)idx[j] * KW4 + c);
-                }
+                ldg_texel<KW4>(levw + (size_t)idx[j] * KW4, tw[j]);
             }
 #pragma unroll
             for (int c = 0; c < KW4; ++c) {
@@ -369,12 +364,7 @@ __device__ __forceinline__ void filtered_w(const ShadeArgs &a, float th, float p
         const float tw[4] = {tp.w00, tp.w01, tp.w10, tp.w11};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if constexpr (KW4 == 2) {  // 32-byte texels in a cudaMalloc'd buffer: every texel is 32-byte aligned
-                ldg8(base + (size_t)idx[j] * 2, t[j][0], t[j][1]);
-            } else {
-#pragma unroll
-                for (int c = 0; c < KW4; ++c) t[j][c] = __ldg(base + (size_t)idx[j] * KW4 + c);
-            }
+            ldg_texel<KW4>(base + (size_t)idx[j] * KW4, t[j]);
         }
 #pragma unroll
         for (int c = 0; c < KW4; ++c) {

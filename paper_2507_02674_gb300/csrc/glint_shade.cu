@@ -30,6 +30,7 @@ namespace {
 // p_k only, one thread per pixel (background 0).
 template <int K, int EV>
 __global__ void __launch_bounds__(kShadeNT) k_probs(ShadeArgs a) {
+    pdl_wait_then_release();
     const long q = (long)blockIdx.x * kShadeNT + threadIdx.x;
     if (q >= a.npix) return;
     const float4 g0 = ldg4(a.view_n0 + q);
@@ -47,6 +48,7 @@ __global__ void __launch_bounds__(kShadeNT) k_probs(ShadeArgs a) {
 
 template <int K, bool INTEGER, bool DEBUG, int EV>
 __global__ void __launch_bounds__(kShadeNT, shade_min_blocks(K)) k_shade(ShadeArgs a) {
+    pdl_wait_then_release();
     const long q = (long)blockIdx.x * kShadeNT + threadIdx.x;
     if (q >= a.npix) return;
     shade_pixel<K, INTEGER, DEBUG, EV>(a, q);
@@ -76,34 +78,31 @@ __global__ void k_quantile(const float *__restrict__ p, float *__restrict__ z, l
     if (i < n) z[i] = normal_quantile(p[i]);
 }
 
+// The kernels of a frame are launched so that their blocks are in place when the
+// stream's previous kernel ends (the map's filter, in a frame whose map has
+// changed).
 template <int K, int EV>
-void launch_ke(const ShadeArgs &args, bool integer, bool debug, cudaStream_t s) {
+cudaError_t launch_ke(const ShadeArgs &args, bool integer, bool debug, cudaStream_t s) {
     const unsigned grid = (unsigned)((args.npix + kShadeNT - 1) / kShadeNT);
-    if (integer) {
-        if (debug) k_shade<K, true, true, EV><<<grid, kShadeNT, 0, s>>>(args);
-        else k_shade<K, true, false, EV><<<grid, kShadeNT, 0, s>>>(args);
-    } else {
-        if (debug) k_shade<K, false, true, EV><<<grid, kShadeNT, 0, s>>>(args);
-        else k_shade<K, false, false, EV><<<grid, kShadeNT, 0, s>>>(args);
-    }
+    return launch_pdl(true,
+                      integer ? (debug ? k_shade<K, true, true, EV> : k_shade<K, true, false, EV>)
+                              : (debug ? k_shade<K, false, true, EV> : k_shade<K, false, false, EV>),
+                      grid, kShadeNT, 0, s, args);
 }
 
 template <int K>
 cudaError_t launch_k(const ShadeArgs &args, bool integer, bool debug, int ev, cudaStream_t s) {
-    if (ev == EV_E2) launch_ke<K, EV_E2>(args, integer, debug, s);
-    else if (ev == EV_GIVEN) launch_ke<K, EV_GIVEN>(args, integer, debug, s);
-    else if (ev == EV_E1A) launch_ke<K, EV_E1A>(args, integer, debug, s);
-    else launch_ke<K, EV_E1>(args, integer, debug, s);
-    return cudaGetLastError();
+    if (ev == EV_E2) return launch_ke<K, EV_E2>(args, integer, debug, s);
+    if (ev == EV_GIVEN) return launch_ke<K, EV_GIVEN>(args, integer, debug, s);
+    if (ev == EV_E1A) return launch_ke<K, EV_E1A>(args, integer, debug, s);
+    return launch_ke<K, EV_E1>(args, integer, debug, s);
 }
 
 template <int K>
 cudaError_t launch_probs(const ShadeArgs &args, int ev, cudaStream_t s) {
     const unsigned grid = (unsigned)((args.npix + kShadeNT - 1) / kShadeNT);
-    if (ev == EV_E2) k_probs<K, EV_E2><<<grid, kShadeNT, 0, s>>>(args);
-    else if (ev == EV_E1A) k_probs<K, EV_E1A><<<grid, kShadeNT, 0, s>>>(args);
-    else k_probs<K, EV_E1><<<grid, kShadeNT, 0, s>>>(args);
-    return cudaGetLastError();
+    return launch_pdl(true, ev == EV_E2 ? k_probs<K, EV_E2> : ev == EV_E1A ? k_probs<K, EV_E1A> : k_probs<K, EV_E1>, grid,
+                      kShadeNT, 0, s, args);
 }
 
 }  // namespace
