@@ -153,18 +153,65 @@ __device__ __forceinline__ float4 lut_fetch(const float4 *lut, int n, float mu, 
 }
 
 
+// The k-th stored weight of a compressed record's code words.
+template <int WFMT>
+__device__ __forceinline__ float decode_w(const uint32_t *words, int k) {
+    if (WFMT == GLINT_WFMT_UNORM8) return (float)((words[k / 4] >> (8 * (k % 4))) & 0xffu) * (1.f / 255.f);
+    const uint32_t h = (words[k / 2] >> (16 * (k % 2))) & 0xffffu;
+    if (WFMT == GLINT_WFMT_F16) return __half2float(__ushort_as_half((unsigned short)h));
+    return (float)h * (1.f / 65535.f);
+}
+
+// Compressed records: adds the four taps' colour and weights, scaled by the
+// level's wl.  Bound by load instructions in flight: each tap's codes come in
+// one load (8 bytes at K = 4, 16 at K = 8, twice 16 at K = 16; half of that for
+// 8-bit codes) and the format is settled once a level, not once a weight
+// (1283 x 717 shading, start to end of frame: K = 8 FP16 143 to 105 us, K = 16
+// UNORM16 348 to 216 us with the packed draws, which alone give 123 to 103 and
+// 349 to 265 us on FP32 maps).
+template <int K, int WFMT, bool NEED_W>
+__device__ __forceinline__ void compressed_taps(const float4 *base, int rec, const Taps &tp, float wl, float4 &rgb,
+                                                float *w) {
+    constexpr int kBytes = K * (WFMT == GLINT_WFMT_UNORM8 ? 1 : 2), kWords = (kBytes + 3) / 4;
+    const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
+    const float tw[4] = {tp.w00, tp.w01, tp.w10, tp.w11};
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t codes[4][kWords];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float4 *r = base + (size_t)idx[t] * rec;
+        v = fma4(tw[t], __ldg(r), v);
+        if (NEED_W) {
+            if constexpr (kWords >= 4) {
+#pragma unroll
+                for (int i = 0; i < kWords; i += 4) {
+                    const uint4 c = __ldg(reinterpret_cast<const uint4 *>(r + 1) + i / 4);
+                    codes[t][i] = c.x; codes[t][i + 1] = c.y; codes[t][i + 2] = c.z; codes[t][i + 3] = c.w;
+                }
+            } else if constexpr (kWords == 2) {
+                const uint2 c = __ldg(reinterpret_cast<const uint2 *>(r + 1));
+                codes[t][0] = c.x; codes[t][1] = c.y;
+            } else {
+                codes[t][0] = __ldg(reinterpret_cast<const uint32_t *>(r + 1));
+            }
+        }
+    }
+    rgb = fma4(wl, v, rgb);
+    if (NEED_W) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float f = wl * tw[t];
+#pragma unroll
+            for (int k = 0; k < K; ++k) w[k] = fmaf(f, decode_w<WFMT>(codes[t], k), w[k]);
+        }
+    }
+}
+
 // Channels (R, G, B, W_1 .. W_K) of the filtered maps at direction (th, ph),
 // bilinear in the levels r0 and r1 blended by ft, into ch[0 .. 3+K) (RGB only
 // unless NEED_W).  FP32 maps hold C4 float4 per texel; compressed ones a
 // record of frec4 x 16 bytes: (R, G, B, -) as float4, then the K weights as
 // FP16, UNORM16 or UNORM8 codes.
-__device__ __forceinline__ float decode_w(uint32_t word, int j, int wfmt) {
-    if (wfmt == GLINT_WFMT_UNORM8) return (float)((word >> (8 * j)) & 0xffu) * (1.f / 255.f);
-    const uint32_t h = (word >> (16 * j)) & 0xffffu;
-    if (wfmt == GLINT_WFMT_F16) return __half2float(__ushort_as_half((unsigned short)h));
-    return (float)h * (1.f / 65535.f);
-}
-
 template <int K, int C4, bool NEED_W>
 __device__ __forceinline__ void filtered_channels(const ShadeArgs &a, float th, float ph, int r0, int r1, float ft,
                                                   float *ch) {
@@ -200,37 +247,21 @@ __device__ __forceinline__ void filtered_channels(const ShadeArgs &a, float th, 
         return;
     }
     // compressed weights
-    const int rec = a.frec4, wfmt = a.wfmt;
-    const int per_word = (wfmt == GLINT_WFMT_UNORM8) ? 4 : 2;
+    const int rec = a.frec4;
     float4 rgb = make_float4(0.f, 0.f, 0.f, 0.f);
     float w[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) w[k] = 0.f;
-#pragma unroll
+#pragma unroll 1
     for (int lv = 0; lv < 2; ++lv) {
         const int2 lev = __ldg(a.flev + (lv ? r1 : r0));
         const int Wr = lev.x, Hr = lev.x / 2;
         const Taps tp = equirect_taps(ph * (kInvTwoPi * (float)Wr) - 0.5f, th * (kInvPi * (float)Hr) - 0.5f, Wr, Hr);
         const float4 *base = a.filt + (size_t)lev.y * rec;
         const float wl = lv ? ft : 1.f - ft;
-        const int idx[4] = {tp.i00, tp.i01, tp.i10, tp.i11};
-        const float tw[4] = {tp.w00, tp.w01, tp.w10, tp.w11};
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int t = 0; t < 4; ++t) v = fma4(tw[t], __ldg(base + (size_t)idx[t] * rec), v);
-        rgb = fma4(wl, v, rgb);
-        if (NEED_W) {
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const uint32_t *codes = reinterpret_cast<const uint32_t *>(base + (size_t)idx[t] * rec + 1);
-                const float f = wl * tw[t];
-#pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const uint32_t word = __ldg(codes + k / per_word);  // same word: loaded once after CSE
-                    w[k] = fmaf(f, decode_w(word, k % per_word, wfmt), w[k]);
-                }
-            }
-        }
+        if (!NEED_W || a.wfmt == GLINT_WFMT_F16) compressed_taps<K, GLINT_WFMT_F16, NEED_W>(base, rec, tp, wl, rgb, w);
+        else if (a.wfmt == GLINT_WFMT_UNORM16) compressed_taps<K, GLINT_WFMT_UNORM16, NEED_W>(base, rec, tp, wl, rgb, w);
+        else compressed_taps<K, GLINT_WFMT_UNORM8, NEED_W>(base, rec, tp, wl, rgb, w);
     }
     ch[0] = rgb.x; ch[1] = rgb.y; ch[2] = rgb.z;
 #pragma unroll

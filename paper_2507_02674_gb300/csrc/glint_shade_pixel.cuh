@@ -120,31 +120,32 @@ __device__ __forceinline__ void draw_integer_pair(uint32_t Na, uint32_t Nb, cons
     nb = (hi2(xi1) < Tb) ? Nb : rb;
 }
 
-// Dual-gated Gaussian (Alg. 1) with real-valued N and counts.
+// Dual-gated Gaussian (Alg. 1) with real-valued N and counts; 0 and 0 at N = 0.
+// Without branches, as draw_integer: the Gaussian of every lane is computed and
+// the gates select (1283 x 717, FP32 maps: K = 4 64.7 us against 75.3 with a branch
+// around empty nodes and one around the Gaussian, K = 16 265 against 349).
 __device__ __forceinline__ void draw_real(float N, const NodeParams &np, uint32_t h1, uint32_t h2, float &n,
                                           float &nbar) {
     const float xi1 = hash_uniform(h1);
-    const float xi1c = hash_uniform_complement(h1);
+    const float xi1c = __fsub_rn(1.f, xi1);
     const float N2 = fmaxf(2.f, N);
-    const float a = fminf(fmaxf(N - 1.f, 0.f), 1.f);
-    const float b = fmaxf(0.f, 1.f - fabsf(1.f - N));
+    const float a = __saturatef(N - 1.f);
+    const float b = __saturatef(1.f - fabsf(1.f - N));
     const float Pall = a * fast_exp2(N2 * np.lp);
     const float Pallneg = a * fast_exp2(N2 * np.lq);
-    const float Pone = b * np.p, Poneneg = b * np.q;
     const bool B_all = xi1 < Pall;
-    const bool B_allone = xi1 < Pall + Pone;
+    const bool B_allone = xi1 < fmaf(b, np.p, Pall);
     const bool B_allneg = xi1c <= Pallneg;
-    const bool B_alloneneg = xi1c <= Pallneg + Poneneg;
+    const bool B_alloneneg = xi1c <= fmaf(b, np.q, Pallneg);
     const bool B_G = (N > 1.f) && !B_allone && !B_alloneneg;
-    float G = 0.f;
-    if (B_G) {
-        const float mu = 1.f + (N2 - 2.f) * np.p;
-        const float sigma = fast_sqrt(fmaxf((N2 - 2.f) * np.p * np.q, 0.f));
-        const float z = normal_quantile(hash_uniform(h2));
-        G = fminf(fmaxf(fmaf(sigma, z, mu), 1.f), N2 - 1.f);
-    }
-    n = (B_all ? N2 - 1.f : 0.f) + (B_allone ? 1.f : 0.f) + G;
-    nbar = (B_allneg ? N2 - 1.f : 0.f) + (B_alloneneg ? 1.f : 0.f) + (B_G ? N2 - G : 0.f);
+    const float m = N2 - 2.f;
+    const float mu = fmaf(m, np.p, 1.f);
+    const float sigma = fast_sqrt(fmaxf(m * np.p * np.q, 0.f));
+    const float z = normal_quantile(hash_uniform(h2));
+    const float N1 = N2 - 1.f;
+    const float g = fminf(fmaxf(fmaf(sigma, z, mu), 1.f), N1);
+    n = (B_all ? N1 : 0.f) + (B_allone ? 1.f : 0.f) + (B_G ? g : 0.f);
+    nbar = (B_allneg ? N1 : 0.f) + (B_alloneneg ? 1.f : 0.f) + (B_G ? N2 - g : 0.f);
 }
 
 
@@ -541,10 +542,8 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
                             h = pcg4d(make_uint4(vx, vy, key2 | ((uint32_t)(1 + n / 2) << 16), a.seed));
                         const uint32_t u1 = (n == 1) ? h.y : (n & 1) ? h.z : h.x;
                         const uint32_t u2 = (n == 1) ? h.z : (n & 1) ? h.w : h.y;
-                        if (N[n] > 0.f) {
-                            if (DRAW == kDrawDual) draw_real(N[n], nd[n], u1, u2, nl, nr);
-                            else draw_single_real(N[n], nd[n], u1, u2, DRAW == kDrawSingleOld, nl, nr);
-                        }
+                        if (DRAW == kDrawDual) draw_real(N[n], nd[n], u1, u2, nl, nr);
+                        else if (N[n] > 0.f) draw_single_real(N[n], nd[n], u1, u2, DRAW == kDrawSingleOld, nl, nr);
                         N[2 * n] = nl;
                         N[2 * n + 1] = nr;
                     }
