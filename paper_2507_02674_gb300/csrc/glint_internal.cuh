@@ -15,12 +15,13 @@ namespace glint {
 // k_shade_var; 128 threads each), their launch bound and the serving grid's
 // unit.  Six blocks give 80 registers a thread: the per-node draw code
 // spills at 64 registers (eight blocks), and a wider budget leaves too few
-// warps to fill the issue slots (1080p frame, K = 8: 0.378 ms at 8 blocks,
-// 0.342 ms at 6, 0.354 ms at 5, 0.403 ms at 4).
+// warps to fill the issue slots (1080p frame, K = 8, with an earlier form of the
+// draws: 0.378 ms at 8 blocks, 0.342 at 6, 0.354 at 5, 0.403 at 4; with the
+// packed draws the map update and frame take 340 us at 6 and 341 at 5).
 constexpr int kShadeMinBlocks = 6;
 // K = 16 (15 draws a pixel, 16-entry arrays) spills 232 bytes at 80
 // registers; four blocks (128 registers) cut that to 40 and the 3840 x 2160
-// grazing frame from 1.393 to 1.320 ms (five blocks: 1.398 ms).
+// grazing frame from 1.393 to 1.320 ms (five blocks: 1.398 ms; scalar draws).
 constexpr int shade_min_blocks(int K) { return K >= 16 ? 4 : kShadeMinBlocks; }
 
 constexpr float kPi = 3.14159265358979323846f;
@@ -318,7 +319,7 @@ cudaError_t glint_launch_serve_mlp(int K, int num_sms, const glint::ShadeArgs *f
                                    int nitems, cudaStream_t s);
 void glint_mlp_weights(const glint_mlp *m, const void **wt, const float **params);
 // Shading with a comparison draw (glint_variants.cu).
-cudaError_t glint_launch_shade_variant(const glint::ShadeArgs &a, int K, bool integer, int draw, int grid,
+cudaError_t glint_launch_shade_variant(const glint::ShadeArgs &a, int K, bool integer, bool debug, int draw, int grid,
                                        cudaStream_t s);
 // Shading with the surrogate fused in (inputs, network and draws in one
 // kernel; p_k stays on chip).

@@ -121,7 +121,8 @@ cudaError_t glint_launch_shade(const glint_ctx *ctx, const glint_env *env, const
     a.pk_in = pk_in;
     if (p->draw != GLINT_DRAW_DUAL || p->grid != GLINT_GRID_ISOTROPIC) {  // comparison draws, anisotropic grid
         if (launches) *launches = a.npix ? 1 : 0;
-        return glint_launch_shade_variant(a, env->d.K, p->count_mode == GLINT_COUNT_INTEGER, p->draw, p->grid, s);
+        return glint_launch_shade_variant(a, env->d.K, p->count_mode == GLINT_COUNT_INTEGER, dbg != nullptr, p->draw,
+                                          p->grid, s);
     }
     const int ev = pk_in ? EV_GIVEN : (p->evaluator == GLINT_EVAL_E2 ? EV_E2
                                        : p->evaluator == GLINT_EVAL_E1_ANISO ? EV_E1A : EV_E1);
