@@ -779,8 +779,10 @@ __device__ __forceinline__ void copy_swz_async(__nv_bfloat16 *dst, const __nv_bf
 // between layers.  So the weights arrive by cp.async, all in flight at once;
 // each warp takes one 16-row tile and half of a layer's outputs; and the column
 // sums (bias gradients) ride along with the last product: six barriers a chunk
-// instead of eleven.  A step of 8192 with the Adam kernel 14.8 -> 12.6 us, of
-// 32768 41.0 -> 32.0, of 517 11.6 -> 9.0.
+// instead of eleven.  Held to 128 registers (168 without a bound above three
+// blocks an SM) although only three blocks an SM are launched: 32 steps of 32768
+// 1023 -> 955 us, of 14591 511 -> 489, of 8192 the same.  A step of 8192 with the
+// Adam kernel 14.8 -> 12.6 us, of 32768 41.0 -> 29.8, of 517 11.6 -> 9.0.
 struct SmemGrad {
     SmemW w;
     SmemWB b;
@@ -795,7 +797,7 @@ struct SmemGrad {
 constexpr int kGradBlocks = 3;
 
 template <int NT>
-__global__ void __launch_bounds__(kNT, kGradBlocks) k_mlp_grad(const uint4 *__restrict__ xg, const float *__restrict__ lpg,
+__global__ void __launch_bounds__(kNT, 4) k_mlp_grad(const uint4 *__restrict__ xg, const float *__restrict__ lpg,
                                                   const float *__restrict__ targets, long n_total, long first,
                                                   long batch, int K, const __nv_bfloat16 *__restrict__ wt,
                                                   const __nv_bfloat16 *__restrict__ wb,
