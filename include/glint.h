@@ -268,8 +268,8 @@ typedef struct glint_debug {
  * anisotropic footprint by an S x S quadrature of the GGX slope distribution
  * reading the weights pyramid (masked mass in p_1), or, with GLINT_EVAL_MLP,
  * p_k from params->mlp evaluated inside the shading kernel (one launch: each
- * block of 256 pixels computes the network's inputs, runs the network on the
- * tensor cores and draws with its p_k from shared memory), or, with
+ * warp computes its 32 pixels' network inputs, runs the network on the tensor
+ * cores and draws with its p_k from shared memory), or, with
  * GLINT_EVAL_GIVEN, the p_k in params->p_scratch,
  * N_P = N_0 |det duv|, and
  * M_k = sum_i w_i n_k(i) over six triangle-grid samples (Sec. 3.3

@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kNT, 4) k_mlp_infer(ShadeArgs a, const __nv_bf
 // us), and warps that share an SM fairly stay in step, so that each phase ran
 // alone: 596 us whatever the occupancy or the barriers.  At K = 8, on frames of
 // several rounds, the two halves of a block therefore take turns (kFusedLarge
-// threads): one computes inputs and network while the other draws.  521 us, 78%
+// threads): one computes inputs and network while the other draws.  520 us, 78%
 // of the L1's throughput and 60% of the issue slots.  (The turn handed over
 // before the network: 544; 640 threads 526, 512 561.)  Smaller frames and K <= 4
 // (16-byte texels, fewer draws) take kFusedNT threads without turns, both of a
@@ -636,16 +636,23 @@ __global__ void __launch_bounds__(NT, 1) k_shade_mlp(ShadeArgs a, const __nv_bfl
     pdl_wait_then_release();
     load_weights<NT>(sm.w, wt, params);
     __syncthreads();
-    // 32-pixel tiles: a block's warps take neighbours (their look-ups share texels)
-    // where a frame gives every warp of the chip one, else the blocks take turns
+    // A round's tiles of 32 pixels go to the blocks in turn, kRun neighbours (their
+    // look-ups share texels) at a time: a block of neighbours only would get the
+    // sky of a frame, or its most expensive rows, whole.  What does not fill a
+    // round goes to all blocks alike, a tile each.  K = 8, 640 x 480 grazing: runs
+    // of one tile 69.4 us, 2 70.5, 4 71.3, 8 72.3, a whole block 78.4; 374 x 280
+    // 29.7, 29.3, 32.4, 32.4, 42.2; 1920 x 1080 525.7, 520.5, 519.8, 521.0, 522.7.
     constexpr bool kTurns = NT == kFusedLarge;
+    constexpr int kRun = 2;
     const int warp = threadIdx.x >> 5, half = warp / (NT / 64);
     const long stride = (long)gridDim.x * NT;  // pixels a round
-    const long tile = a.npix >= stride ? (long)blockIdx.x * (NT / 32) + warp : (long)warp * gridDim.x + blockIdx.x;
     const long rounds = (a.npix + stride - 1) / stride;  // the same for every warp
     if (kTurns && half == 1) half_arrive(1, NT);         // the first half begins
 #pragma unroll 1
     for (long i = 0; i < rounds; ++i) {
+        const long left = a.npix - i * stride;
+        const int run = left >= stride ? kRun : 1;
+        const long tile = ((long)(warp / run) * gridDim.x + blockIdx.x) * run + warp % run;
         const long q = i * stride + tile * 32 + (threadIdx.x & 31);
         const bool valid = q < a.npix;
         float4 g0;
