@@ -592,7 +592,9 @@ int glint_plan_tick(long *next, const long *npix, int nframes, long tick_pixels,
 /* Standard normal quantile z = Phi^-1(p) as the shading kernel evaluates it for
  * the Gaussian part of the dual-gated draw (Alg. 1): for n device floats p in
  * (0, 1), device output z.  Relative error below 2.3e-7 on the uniforms the
- * kernel draws, p = (2m + 1) 2^-24 (FP32).  Enqueued on `stream`. */
+ * kernel draws, p = (2m + 1) 2^-24 (FP32), and below 2^-20 for any p from 2^-25
+ * on (2^-22 absolute for |z| < 1/4); smaller p are extrapolated (1e-6 relative at
+ * 1e-8, 3e-4 at 1e-10).  Enqueued on `stream`. */
 glint_status glint_normal_quantile(const float *p, float *z, long n, void *stream);
 
 /* Fixed scratch of glint_env_levels_noalloc: one (min, max) float pair per

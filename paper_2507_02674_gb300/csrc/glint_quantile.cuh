@@ -10,19 +10,25 @@
 // (the hardware lg2, no conversion), and the factor sqrt(2) is part of the
 // polynomials: Phi^-1(p) = x Q1(w2 - c1) for w2 < 5 / ln 2, else
 // x Q2(sqrt(w2) - c2), Q1 and Q2 of degree 9 with coefficients fitted for
-// this library by weighted least squares against the exact quantile.  For the
-// uniforms the hash produces, p = (2m + 1) 2^-24, x is exact in FP32 and
-// 4p - 4p^2 is rounded once (one fused multiply-add); lg2's error moves Q1 by
-// less than 3e-8 relative; the result stays within 2.5e-7 relative (4.2e-8
-// absolute for |z| < 1/4) of the exact quantile.
+// this library by weighted least squares against the exact quantile, for
+// p in [2^-25, 1 - 2^-25].  There are two forms of the logarithm's argument, each
+// one fused multiply-add:
+//   4p - 4p^2  for any p (normal_quantile): accurate where x = 2p - 1 rounds;
+//   1 - x^2    for the uniforms the hash produces, p = (2m + 1) 2^-24
+//              (hash_quantile, hash_quantile2): x is exact in FP32 there, so both
+//              round the same number, and this one is an operation shorter.
+// lg2's error moves Q1 by less than 3e-8 relative; on those uniforms the result
+// stays within 2.5e-7 relative (4.2e-8 absolute for |z| < 1/4) of the exact
+// quantile.  Below 2^-25 Q2 is extrapolated (1e-6 relative at p = 1e-8, 3e-4 at
+// 1e-10).
 #pragma once
 
 namespace glint {
 
-__device__ __forceinline__ float normal_quantile(float p) {
-    const float x = 2.f * p - 1.f;
+// Phi^-1(p) from x = 2p - 1 and v = 4p (1 - p) = 1 - x^2.
+__device__ __forceinline__ float quantile_of(float x, float v) {
     float w2;
-    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(w2) : "f"(fmaf(-x, x, 1.f)));
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(w2) : "f"(v));
     w2 = -w2;
     float P;
     if (w2 < 7.213475227f) {
@@ -55,9 +61,21 @@ __device__ __forceinline__ float normal_quantile(float p) {
     return P * x;
 }
 
-// normal_quantile of two arguments in packed FP32, the same results.  The tail
+// Any p in (0, 1).
+__device__ __forceinline__ float normal_quantile(float p) {
+    const float p4 = 4.f * p;
+    return quantile_of(2.f * p - 1.f, fmaf(-p4, p, p4));
+}
+
+// p = (2m + 1) 2^-24, a uniform of the hash: normal_quantile's result.
+__device__ __forceinline__ float hash_quantile(float p) {
+    const float x = 2.f * p - 1.f;
+    return quantile_of(x, fmaf(-x, x, 1.f));
+}
+
+// hash_quantile of two arguments in packed FP32, the same results.  The tail
 // (0.35% of the uniforms) is evaluated for both when either needs it.
-__device__ __forceinline__ f32x2 normal_quantile2(f32x2 p) {
+__device__ __forceinline__ f32x2 hash_quantile2(f32x2 p) {
     const f32x2 x = fma2(pack2(2.f, 2.f), p, pack2(-1.f, -1.f));
     const f32x2 v = fma2(mul2(x, pack2(-1.f, -1.f)), x, pack2(1.f, 1.f));
     float wa, wb;

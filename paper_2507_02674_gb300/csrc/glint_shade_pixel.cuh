@@ -82,7 +82,7 @@ __device__ __forceinline__ uint32_t draw_integer(uint32_t N, const NodeParams &n
     const float Sneg = fast_exp2(Nf * np.lq);
     const float muh = fmaf(m, np.p, 1.5f);
     const float sigma = fast_sqrt(m * np.p * np.q);
-    const float z = normal_quantile(hash_uniform(h2));
+    const float z = hash_quantile(hash_uniform(h2));
     const float G = fmaxf(fmaf(sigma, z, muh), 1.f);
     uint32_t r = min(__float2uint_rz(G), N - 1u);  // saturates above 2^32
     r = (xi1c <= Sneg) ? 0u : r;
@@ -110,7 +110,7 @@ __device__ __forceinline__ void draw_integer_pair(uint32_t Na, uint32_t Nb, cons
     const f32x2 muh = fma2(m, np.p, pack2(1.5f, 1.5f));
     const f32x2 var = mul2(mul2(m, np.p), np.q);
     const f32x2 sigma = pack2(fast_sqrt(lo2(var)), fast_sqrt(hi2(var)));
-    const f32x2 z = normal_quantile2(hash_uniform2(h.y, h.w));
+    const f32x2 z = hash_quantile2(hash_uniform2(h.y, h.w));
     const f32x2 g = fma2(sigma, z, muh);
     uint32_t ra = min(__float2uint_rz(fmaxf(lo2(g), 1.f)), Na - 1u);
     uint32_t rb = min(__float2uint_rz(fmaxf(hi2(g), 1.f)), Nb - 1u);
@@ -141,7 +141,7 @@ __device__ __forceinline__ void draw_real(float N, const NodeParams &np, uint32_
     const float m = N2 - 2.f;
     const float mu = fmaf(m, np.p, 1.f);
     const float sigma = fast_sqrt(fmaxf(m * np.p * np.q, 0.f));
-    const float z = normal_quantile(hash_uniform(h2));
+    const float z = hash_quantile(hash_uniform(h2));
     const float N1 = N2 - 1.f;
     const float g = fminf(fmaxf(fmaf(sigma, z, mu), 1.f), N1);
     n = (B_all ? N1 : 0.f) + (B_allone ? 1.f : 0.f) + (B_G ? g : 0.f);
@@ -231,7 +231,7 @@ __device__ __forceinline__ uint32_t draw_single_integer(uint32_t N, const NodePa
     if (N == 1u) return 1u;
     const float mu = 1.f + (Nf - 1.f) * np.p;
     const float sigma = fast_sqrt((Nf - 1.f) * np.p * np.q);
-    const float z = normal_quantile(hash_uniform(h2));
+    const float z = hash_quantile(hash_uniform(h2));
     const float g = fmaf(sigma, z, mu);
     float G = old ? floorf(g) : floorf(g + 0.5f);
     G = fminf(fmaxf(G, 1.f), Nf);
@@ -251,7 +251,7 @@ __device__ __forceinline__ void draw_single_real(float N, const NodeParams &np, 
     if (open) {
         const float mu = 1.f + (N - 1.f) * np.p;
         const float sigma = fast_sqrt(fmaxf((N - 1.f) * np.p * np.q, 0.f));
-        const float z = normal_quantile(hash_uniform(h2));
+        const float z = hash_quantile(hash_uniform(h2));
         const float g = fminf(fmaxf(fmaf(sigma, z, mu), 1.f), fmaxf(N, 1.f));
         n = old ? floorf(g) : g;
     }
