@@ -152,7 +152,8 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
         sincospif(2.f * ((float)i + 0.5f) / (float)S, &sp, &cp);
         angle[i] = make_float2(cp, sp);
     }
-    pdl_wait_then_release();
+    pdl_wait();
+    if (a.npix <= 128L * kFewBlocks) pdl_release();  // as the kernels of a thread a pixel do
     const long q0 = ((long)blockIdx.x * kWarps + warp) * ppw;
     if (lane < ppw) {
         E2Pixel e;

@@ -275,6 +275,19 @@ __device__ __forceinline__ void pdl_wait_then_release() {
     pdl_wait();
     pdl_release();
 }
+// For kernels whose blocks fill a good part of the chip: the release is left to the
+// blocks' ends.  The next kernel's blocks hold the places that they are given while
+// they wait, so blocks scheduled early crowd the SMs that drain first; a grid
+// of about half a wave to one wave then runs unevenly (E2 by a thread a pixel, S =
+// 16, in calls in a row: 320 x 240, K = 2 168 us with an ordinary launch, 253
+// released at once, 166 at the end; K = 8 242, 332, 239; E1's multi-tap p_k, K = 8
+// 14.5, 19.8, 12.7).  At most a block an SM crowds nothing, and takes the launch
+// out of the way of calls of a few microseconds (64 x 64: 8.8 against 9.2 us).
+constexpr unsigned kFewBlocks = 152;
+__device__ __forceinline__ void pdl_wait_then_release_few() {
+    pdl_wait();
+    if (gridDim.x <= kFewBlocks) pdl_release();
+}
 
 // A launch whose blocks may start while the stream's previous kernel runs
 // (pdl), or an ordinary one.

@@ -30,7 +30,7 @@ namespace {
 // p_k only, one thread per pixel (background 0).
 template <int K, int EV>
 __global__ void __launch_bounds__(kShadeNT) k_probs(ShadeArgs a) {
-    pdl_wait_then_release();
+    pdl_wait_then_release_few();
     const long q = (long)blockIdx.x * kShadeNT + threadIdx.x;
     if (q >= a.npix) return;
     const float4 g0 = ldg4(a.view_n0 + q);
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kShadeNT) k_probs(ShadeArgs a) {
 
 template <int K, bool INTEGER, bool DEBUG, int EV>
 __global__ void __launch_bounds__(kShadeNT, shade_min_blocks(K)) k_shade(ShadeArgs a) {
-    pdl_wait_then_release();
+    pdl_wait_then_release_few();
     const long q = (long)blockIdx.x * kShadeNT + threadIdx.x;
     if (q >= a.npix) return;
     shade_pixel<K, INTEGER, DEBUG, EV>(a, q);

@@ -14,7 +14,7 @@ namespace {
 
 template <int K, bool INTEGER, bool DEBUG, int DRAW, int GRID>
 __global__ void __launch_bounds__(kShadeNT, shade_min_blocks(K)) k_shade_var(ShadeArgs a) {
-    pdl_wait_then_release();
+    pdl_wait_then_release_few();
     const long q = (long)blockIdx.x * kShadeNT + threadIdx.x;
     if (q >= a.npix) return;
     shade_pixel<K, INTEGER, DEBUG, EV_E1, DRAW, GRID>(a, q);
