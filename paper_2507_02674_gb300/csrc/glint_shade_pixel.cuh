@@ -3,6 +3,8 @@
 // single-gated forms Eq. gated / Eq. oldgated, and the hierarchical
 // multinomial).  See glint_shade.cu for the per-pixel steps.
 #pragma once
+#include <type_traits>
+
 #include "glint_internal.cuh"
 #include "glint_probs.cuh"
 #include "glint_quantile.cuh"
@@ -122,8 +124,10 @@ __device__ __forceinline__ void draw_integer_pair(uint32_t Na, uint32_t Nb, cons
 
 // Dual-gated Gaussian (Alg. 1) with real-valued N and counts; 0 and 0 at N = 0.
 // Without branches, as draw_integer: the Gaussian of every lane is computed and
-// the gates select (1283 x 717, FP32 maps: K = 4 64.7 us against 75.3 with a branch
-// around empty nodes and one around the Gaussian, K = 16 265 against 349).
+// the gates select (1283 x 717, FP32 maps, ground plane and spheres: K = 4 62 us
+// against 70 with a branch around empty nodes and one around the Gaussian, K = 16
+// 257 against 340; with the Gaussians of two siblings behind one branch 64 and
+// 292).
 __device__ __forceinline__ void draw_real(float N, const NodeParams &np, uint32_t h1, uint32_t h2, float &n,
                                           float &nbar) {
     const float xi1 = hash_uniform(h1);
@@ -146,6 +150,19 @@ __device__ __forceinline__ void draw_real(float N, const NodeParams &np, uint32_
     const float g = fminf(fmaxf(fmaf(sigma, z, mu), 1.f), N1);
     n = (B_all ? N1 : 0.f) + (B_allone ? 1.f : 0.f) + (B_G ? g : 0.f);
     nbar = (B_allneg ? N1 : 0.f) + (B_alloneneg ? 1.f : 0.f) + (B_G ? N2 - g : 0.f);
+}
+
+// draw_real for N <= 1, where only the gates of one trial are left: the same
+// results.  A tree whose root has at most one trial has no other node (a count is
+// 0 or 1), so that distant or sparse surfaces need none of the Gaussians (a sphere
+// of 1283 x 717 pixels, 0.2 microfacets a pixel, K = 4, 8, 16: 37, 54, 99 us, all
+// nodes by draw_real 52, 98, 213, with its Gaussian behind a branch 43, 71, 150).
+__device__ __forceinline__ void draw_real_sparse(float N, const NodeParams &np, uint32_t h1, float &n, float &nbar) {
+    const float xi1 = hash_uniform(h1);
+    const float xi1c = __fsub_rn(1.f, xi1);
+    const float b = __saturatef(1.f - fabsf(1.f - N));
+    n = xi1 < __fmul_rn(b, np.p) ? 1.f : 0.f;
+    nbar = xi1c <= __fmul_rn(b, np.q) ? 1.f : 0.f;
 }
 
 
@@ -434,6 +451,8 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
     float M[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) M[k] = 0.f;
+    // real counts: whether a lane of the warp has more than one trial (either tree gives the same counts)
+    const bool dense = !INTEGER && DRAW == kDrawDual && __any_sync(__activemask(), NP > 1.f);
     const float F2 = 0x1.76cf5ep-2f;  // (sqrt(3) - 1) / 2
     const float fN = floorf(NP);
     const float fracN = NP - fN;
@@ -534,6 +553,28 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
 #pragma unroll
                     for (int n = 2; n < 2 * K; ++n) N[n] = 0.f;
                     draw_single_real(N[1], nd[1], h.y, h.z, false, N[K], N[K + 1]);
+                } else if (DRAW == kDrawDual) {
+                    auto tree = [&](auto draw, auto skip) {  // skip: a pair without trials in any lane of the warp
+                        draw(N[1], nd[1], h.y, h.z, N[2], N[3]);
+#pragma unroll
+                        for (int m = 1; m < K / 2; ++m) {
+                            N[4 * m] = N[4 * m + 1] = N[4 * m + 2] = N[4 * m + 3] = 0.f;
+                            if (!skip.value || N[2 * m] > 0.f || N[2 * m + 1] > 0.f) {
+                                h = pcg4d(make_uint4(vx, vy, key2 + ((uint32_t)(1 + m) << 16), a.seed));
+                                draw(N[2 * m], nd[2 * m], h.x, h.y, N[4 * m], N[4 * m + 1]);
+                                draw(N[2 * m + 1], nd[2 * m + 1], h.z, h.w, N[4 * m + 2], N[4 * m + 3]);
+                            }
+                        }
+                    };
+                    if (dense) {
+                        tree([](float n, const NodeParams &np, uint32_t h1, uint32_t h2, float &l, float &r) {
+                            draw_real(n, np, h1, h2, l, r);
+                        }, std::integral_constant<bool, (K >= 8)>{});
+                    } else {
+                        tree([](float n, const NodeParams &np, uint32_t h1, uint32_t, float &l, float &r) {
+                            draw_real_sparse(n, np, h1, l, r);
+                        }, std::true_type{});
+                    }
                 } else {
 #pragma unroll
                     for (int n = 1; n < K; ++n) {
@@ -542,8 +583,7 @@ __device__ __forceinline__ void shade_draws(const ShadeArgs &a, long q, const fl
                             h = pcg4d(make_uint4(vx, vy, key2 | ((uint32_t)(1 + n / 2) << 16), a.seed));
                         const uint32_t u1 = (n == 1) ? h.y : (n & 1) ? h.z : h.x;
                         const uint32_t u2 = (n == 1) ? h.z : (n & 1) ? h.w : h.y;
-                        if (DRAW == kDrawDual) draw_real(N[n], nd[n], u1, u2, nl, nr);
-                        else if (N[n] > 0.f) draw_single_real(N[n], nd[n], u1, u2, DRAW == kDrawSingleOld, nl, nr);
+                        if (N[n] > 0.f) draw_single_real(N[n], nd[n], u1, u2, DRAW == kDrawSingleOld, nl, nr);
                         N[2 * n] = nl;
                         N[2 * n + 1] = nr;
                     }
