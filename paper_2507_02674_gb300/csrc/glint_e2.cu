@@ -1,22 +1,35 @@
 // E2 reflection probabilities p_k alone (Eq. probhk by quadrature; the points,
-// weights and pyramid level of e2_probabilities in glint_probs.cuh), a warp a
-// pixel.  The surrogate's labels, and the reference its error is judged by.
+// weights and pyramid level of e2_probabilities in glint_probs.cuh), 32 or 8 lanes
+// a pixel.  The surrogate's labels, and the reference its error is judged by.
 //
 // What bounds it: the L1's look-ups of lines and banks.  A point reads 2 x 2
-// texels of 32 bytes (K = 8) at a direction of its own.  One thread a pixel took
-// 22 wavefronts a request, 88 for 32 points (1280 x 720, S = 32: 9.15 ms at 95%
-// of the L1's throughput).  Here the lanes of a warp take points of one pixel,
-// eight in a row along the lobe's radius (the closest on the map) a request,
-// and four adjacent lanes share their four points: in each of four requests a
-// quad reads the 2 x 2 texels of one point, which the swapped columns of the
-// pyramid's odd rows (pyr_column) put in four different banks.  The lanes
-// exchange two words a point for it (texel and weight) and each accumulates
-// what it reads; the sums meet at the end of the pixel.  5.78 ms: 80% of the
-// L1's wavefronts, 74% of the issue slots, 62% of the L2's throughput.  Two
-// lanes a point took 7.3 ms; a request over every fourth ring instead of eight
-// in a row 6.6; words exchanged through shared memory 7.4; blocks of
-// 12 or 24 warps in step, which double the L1's hits, 6.3 and 6.5; without the
-// branch over invalid points 6.9.
+// texels of 32 bytes (K = 8) at a direction of its own; one thread a pixel makes
+// 32 unrelated look-ups a request where neighbouring pixels differ (their
+// roughness, their normal).  Here the lanes take points of one pixel, in a row
+// along the lobe's radius (the closest on the map) in each request, and four
+// adjacent lanes share their four points: in each of four requests a quad reads
+// the 2 x 2 texels of one point, which the swapped columns of the pyramid's odd
+// rows (pyr_column) put in four different banks.  The lanes exchange two words a
+// point for it (texel and weight) and each accumulates what it reads; the sums
+// meet at the end of the pixel.
+//
+// 32 lanes a pixel serve many points (a request takes eight in a row), and frames
+// too small to fill the chip otherwise.  8 lanes a pixel, four neighbouring
+// pixels at a time, waste fewer lanes at the end of few points, share the set-up
+// and the final sums, and read the same lines where neighbouring pixels look the
+// same way, as a thread a pixel does.  1280 x 720, us, thread / 8 lanes / 32 lanes;
+// "rough": random roughness a pixel, "smooth": one sphere, one roughness:
+//   K = 4,  S = 16 rough 1599 / 1383 / 1466, smooth 1124 / 1071 / 1151
+//   K = 8,  S = 13 rough 1476 / 1145 / 1397, smooth 828 / 862 / 1021
+//           S = 16 rough 2263 / 1597 / 1710, smooth 1267 / 1212 / 1446
+//           S = 32 rough 9080 / 6050 / 5802, smooth 5106 / 4617 / 4706
+//   K = 16, S = 8  rough 1303 / 820 / 1090, smooth 467 / 568 / 743
+//           S = 16 rough 5305 / 2967 / 3225, smooth 1858 / 1950 / 2622
+// (K = 8, S = 32, 32 lanes: two lanes a point took 7.3 ms; a request over every
+// fourth ring instead of eight in a row 6.6; words exchanged through shared
+// memory 7.4; blocks of 12 or 24 warps in step 6.3 and 6.5; without the branch over
+// invalid points 6.9.  The sums of 8 lanes in the order of 32, so that both give the
+// same bits: K = 8, S = 13, smooth 977 us.)
 #include "glint_internal.cuh"
 #include "glint_probs.cuh"
 
@@ -25,7 +38,7 @@ using namespace glint;
 namespace {
 
 constexpr int kWarps = 4;       // warps a block
-constexpr int kMaxPpw = 8;      // pixels a warp at most (their geometry is staged by as many lanes at once)
+constexpr int kMaxSteps = 8;    // pixels a group of lanes takes one after the other at most
 constexpr int kMaxS = 256;
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -87,13 +100,15 @@ struct __align__(16) E2Pixel {
     int pad[2];
 };
 
-// Sum of v[0 .. K) over the warp: lane L ends with the sum of v[L >> (5 - log2 K)].
-template <int K>
-__device__ __forceinline__ float warp_sums(float (&v)[K]) {
+// Sums of v[0 .. K) over groups of G lanes: with K <= G, lane L of a group ends with
+// the sum of v[L >> (log2 G - log2 K)] in v[0], else with those of v[L K / G ..] in
+// v[0 .. K / G).
+template <int K, int G>
+__device__ __forceinline__ void group_sums(float (&v)[K]) {
     const int lane = threadIdx.x & 31;
     int n = K;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    for (int o = G / 2; o > 0; o >>= 1) {
         if (n > 1) {
             n /= 2;
             const bool up = lane & o;
@@ -107,7 +122,6 @@ __device__ __forceinline__ float warp_sums(float (&v)[K]) {
             v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
         }
     }
-    return v[0];
 }
 
 // acc += w (texel idx), the weights of the texel's components.  With 64-byte
@@ -134,16 +148,21 @@ __device__ __forceinline__ void add_texel(const float4 *__restrict__ lev, unsign
     }
 }
 
-// FIXED: S is a power of two from 8, so that a lane keeps its ring(s) of points.
-template <int K, bool FIXED>
-__global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int ppw) {
-    constexpr int KW4 = (3 + K + 3) / 4 - 1;
+// G lanes (32 or 8) a pixel, so 32 / G pixels a warp at a time.  FIXED: S is a power
+// of two from 8, so that a lane keeps its ring(s) of points.  Five blocks an SM;
+// six (80 registers) where it is faster (8 lanes, rough, K = 8: S = 16 1705 -> 1597 us,
+// but S = 24 3515 -> 3596; K = 16: S = 16 3116 -> 2967, S = 24 7020 -> 6687).
+template <int K, bool FIXED, int G>
+__global__ void __launch_bounds__(kWarps * 32, G == 8 && (FIXED || K == 16) ? 6 : 5) k_e2_probs(ShadeArgs a, int steps) {
+    constexpr int KW4 = (3 + K + 3) / 4 - 1, kGroups = 32 / G, kMaxPpw = kGroups * kMaxSteps;
+    static_assert(kMaxPpw <= 32, "a warp's pixels are staged by a lane each");
     __shared__ float2 ring[kMaxS];   // r, 2 s
     __shared__ float2 angle[kMaxS];  // cos, sin
     __shared__ E2Pixel px[kWarps][kMaxPpw];
     const int S = a.e2S, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // the lane's place in a step's 32 points: a request takes eight in a row (one of each quad)
-    const int lp = (lane >> 2) + 8 * (lane & 3);
+    const int ppw = kGroups * steps, group = lane / G;
+    // the lane's place in a step's G points: a request takes G / 4 in a row (one of each quad)
+    const int lp = ((lane % G) >> 2) + (G / 4) * (lane & 3);
     const bool right = lane & 1, lower = lane & 2;  // the texel of a look-up that this lane reads
     for (int i = threadIdx.x; i < S; i += kWarps * 32) {
         const float sv = ((float)i + 0.5f) / (float)S;
@@ -186,17 +205,20 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
     }
     __syncthreads();
 #pragma unroll 1
-    for (int j = 0; j < ppw; ++j) {
-        const long q = q0 + j;
-        if (q >= a.npix) return;
-        const E2Pixel e = px[warp][j];
-        if (e.level < 0) {
-            if (lane < K) a.p_out[q * K + lane] = 0.f;
+    for (int j = 0; j < ppw; j += kGroups) {
+        const long q = q0 + j + group;
+        if (q0 + j >= a.npix) return;
+        const E2Pixel e = px[warp][j + group];
+        const bool live = e.level >= 0;  // (past the end of the frame: no)
+        if (G == 32 ? !live : !__any_sync(0xffffffffu, live)) {
+            if (q < a.npix)
+                for (int k = lane % G; k < K; k += G) a.p_out[q * K + k] = 0.f;
             continue;
         }
-        const int W = a.envW >> e.level, H = a.envH >> e.level;
+        const int level = max(e.level, 0);
+        const int W = a.envW >> level, H = a.envH >> level;
         const float Wf = (float)W, Hf = (float)H;
-        const float4 *lev = a.pyr + a.pyr_w4[e.level];
+        const float4 *lev = a.pyr + a.pyr_w4[level];
         float acc[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) acc[k] = 0.f;
@@ -213,7 +235,7 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
             const float wgt = s2 * sqrt_approx(hl2);
             sum_all += wgt;
             sum_inv += valid ? 0.f : wgt;
-            const float w = valid ? wgt : 0.f;
+            const float w = valid && (G == 32 || live) ? wgt : 0.f;  // background beside a live pixel reads nothing
             const float c = 2.f * oh * rcp_approx(hl2);
             const float hx = e.nx - sx * e.tx - sy * e.bx;
             const float hy = e.ny - sx * e.ty - sy * e.by;
@@ -251,17 +273,17 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
             add_texel<K, KW4>(lev, lower ? j1 : j3, lower ? g1 : g3, lower, acc);
         };
         if (FIXED) {
-            const int per = max(32 / S, 1);  // angles at a time
-            for (int g = 0; g < S; g += 32) {
+            const int per = max(G / S, 1);  // angles at a time
+            for (int g = 0; g < S; g += G) {
                 const float2 rs = ring[(lp & (S - 1)) + g];
                 const float axr = e.ax * rs.x, ayr = e.ay * rs.x;
 #pragma unroll 1
-                for (int ic = S < 32 ? lp / S : 0; ic < S; ic += per) point(axr, ayr, rs.y, angle[ic]);
+                for (int ic = S < G ? lp / S : 0; ic < S; ic += per) point(axr, ayr, rs.y, angle[ic]);
             }
         } else {
             int ia = lp % S, ic = lp / S;
-            const int da = 32 % S, dc = 32 / S;
-            for (int i = lp; i - lp < S * S; i += 32) {  // the same trips for every lane
+            const int da = G % S, dc = G / S;
+            for (int i = lp; i - lp < S * S; i += G) {  // the same trips for every lane
                 const bool in = i < S * S;
                 const float2 rs = ring[ia];
                 point(e.ax * rs.x, e.ay * rs.x, in ? rs.y : 0.f, angle[in ? ic : 0]);
@@ -271,7 +293,7 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
             }
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = G / 2; o > 0; o >>= 1) {
             sum_all += __shfl_xor_sync(0xffffffffu, sum_all, o);
             sum_inv += __shfl_xor_sync(0xffffffffu, sum_inv, o);
         }
@@ -283,33 +305,45 @@ __global__ void __launch_bounds__(kWarps * 32, 5) k_e2_probs(ShadeArgs a, int pp
                 acc[k + K / 2] = t;
             }
         }
-        constexpr int kPer = 32 / K;  // lanes that hold the same sum
-        const float v = warp_sums<K>(acc);
-        const int k = lane / kPer;
-        if (lane % kPer == 0) a.p_out[q * K + k] = (k == 0 ? sum_inv + v : v) / sum_all;
+        group_sums<K, G>(acc);
+        constexpr int kPer = G >= K ? G / K : 1, kOwn = G >= K ? 1 : K / G;  // lanes that hold the same sum, sums a lane
+        if (q < a.npix && lane % G % kPer == 0) {
+#pragma unroll
+            for (int i = 0; i < kOwn; ++i) {
+                const int k = lane % G / kPer * kOwn + i;
+                a.p_out[q * K + k] = live ? (k == 0 ? sum_inv + acc[i] : acc[i]) / sum_all : 0.f;
+            }
+        }
     }
 }
 
-template <int K>
+template <int K, int G>
 cudaError_t launch(const ShadeArgs &a, int num_sms, cudaStream_t s) {
-    // several pixels a warp once there are warps enough without
+    // several pixels a group once there are warps enough without
     const long want = (long)num_sms * 24 * 4;
-    int ppw = kMaxPpw;
-    while (ppw > 1 && a.npix / ppw < want) ppw >>= 1;
-    const long per_block = (long)kWarps * ppw;
+    constexpr int kGroups = 32 / G;
+    int steps = kMaxSteps;
+    while (steps > 1 && a.npix / (kGroups * steps) < want) steps >>= 1;
+    const long per_block = (long)kWarps * kGroups * steps;
     const unsigned grid = (unsigned)((a.npix + per_block - 1) / per_block);
     const bool fixed = a.e2S >= 8 && (a.e2S & (a.e2S - 1)) == 0;
-    return launch_pdl(true, fixed ? k_e2_probs<K, true> : k_e2_probs<K, false>, grid, kWarps * 32, 0, s, a, ppw);
+    auto kernel = k_e2_probs<K, true, G>;
+    if constexpr (K >= 8 || G == 32) {  // (8 lanes take K <= 4 only with a power of two)
+        if (!fixed) kernel = k_e2_probs<K, false, G>;
+    } else if (!fixed) {
+        return cudaErrorInvalidValue;
+    }
+    return launch_pdl(true, kernel, grid, kWarps * 32, 0, s, a, steps);
 }
 
 }  // namespace
 
-cudaError_t glint_launch_e2_probs(const ShadeArgs &a, int K, int num_sms, cudaStream_t s) {
+cudaError_t glint_launch_e2_probs(const ShadeArgs &a, int K, int lanes, int num_sms, cudaStream_t s) {
     switch (K) {
-    case 2: return launch<2>(a, num_sms, s);
-    case 4: return launch<4>(a, num_sms, s);
-    case 8: return launch<8>(a, num_sms, s);
-    case 16: return launch<16>(a, num_sms, s);
+    case 2: return lanes == 8 ? launch<2, 8>(a, num_sms, s) : launch<2, 32>(a, num_sms, s);
+    case 4: return lanes == 8 ? launch<4, 8>(a, num_sms, s) : launch<4, 32>(a, num_sms, s);
+    case 8: return lanes == 8 ? launch<8, 8>(a, num_sms, s) : launch<8, 32>(a, num_sms, s);
+    case 16: return lanes == 8 ? launch<16, 8>(a, num_sms, s) : launch<16, 32>(a, num_sms, s);
     default: return cudaErrorInvalidValue;
     }
 }

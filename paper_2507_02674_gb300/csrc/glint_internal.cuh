@@ -338,8 +338,8 @@ cudaError_t glint_launch_shade_variant(const glint::ShadeArgs &a, int K, bool in
 // kernel; p_k stays on chip).
 cudaError_t glint_launch_shade_mlp(const glint_ctx *ctx, const glint_env *env, const glint_gbuffer *g,
                                    const glint_params *p, float *out, const glint_debug *dbg, cudaStream_t s);
-// p_k of the E2 quadrature alone, a warp a pixel (glint_e2.cu).
-cudaError_t glint_launch_e2_probs(const glint::ShadeArgs &a, int K, int num_sms, cudaStream_t s);
+// p_k of the E2 quadrature alone, 8 or 32 lanes a pixel (glint_e2.cu).
+cudaError_t glint_launch_e2_probs(const glint::ShadeArgs &a, int K, int lanes, int num_sms, cudaStream_t s);
 // p_k only (E1 or E2), background pixels 0.
 cudaError_t glint_launch_probs(const glint_ctx *ctx, const glint_env *env, const glint_gbuffer *g,
                                const glint_params *p, float *p_out, cudaStream_t s);

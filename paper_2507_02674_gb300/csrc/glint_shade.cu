@@ -142,20 +142,23 @@ cudaError_t glint_launch_shade(const glint_ctx *ctx, const glint_env *env, const
     return e;
 }
 
-// A warp a pixel (glint_e2.cu) or a thread a pixel for E2's p_k.  The warp's
-// points fill whole steps of 32 and pay for its set-up and final sums only from
-// some S on, sooner the more a point reads (1280 x 720, us, thread / warp; K = 2:
-// S = 14 1127 / 1223, S = 16 1467 / 1296, S = 24 3275 / 2905; K = 4: S = 16 1606 /
-// 1430; K = 8: S = 10 879 / 1000, S = 12 1280 / 1198, S = 32 9150 / 5780; K = 16:
-// S = 6 916 / 862, S = 16 7381 / 3230); steps are shorter where S is a power of
-// two.  Frames that leave most of the chip without a thread of its own take the
-// warp from S = 5 on (14400 pixels, S = 5: 22 / 14; 19200, K = 2, S = 4: 12 / 14;
-// 57600, S = 6: 35 / 50).
-static bool e2_by_warps(int K, int S, long npix, int num_sms) {
-    if (S >= 5 && npix <= 128L * num_sms) return true;
-    if (K == 16) return S >= 6;
-    if (K == 8) return S >= 12;
-    return S >= 24 || S == 16;
+// Lanes a pixel for E2's p_k: 8 or 32 (glint_e2.cu), or 1 (k_probs), by K and S.
+// Several lanes pay for their set-up and final sums from some S on, sooner the more
+// a point reads and the less neighbouring pixels read the same lines (1280 x 720,
+// thread / 8 lanes, us, rough and smooth frames of glint_e2.cu: K = 4, S = 8 401 / 384,
+// 297 / 288, S = 17 1810 / 1635, 1266 / 1306; K = 8, S = 11 1048 / 855, 600 / 645, S = 12
+// 1255 / 955, 710 / 719; K = 16, S = 7 986 / 705, 349 / 423, S = 8 1303 / 820, 467 /
+// 568).  For K <= 4 only a power of two, whose steps are whole, pays below 24.  Above
+// S = 20 small frames lose more by 8 lanes than large ones gain (K = 8, S = 24, 8 / 32
+// lanes: 64 x 64 43 / 24 us, 1280 x 720 3514 / 3598; S = 16 21 / 14, 1597 / 1710).
+// Below those S frames that leave most of the chip without a thread of its own
+// take 32 lanes (160 x 120, K = 8, thread / 32 lanes: S = 4 15 / 16 us, S = 5 22 / 17, S = 11
+// 93 / 30).  The splits differ in rounding.
+static int e2_lanes(int K, int S, long npix, int num_sms) {
+    const bool pow2 = (S & (S - 1)) == 0;
+    const int from = K == 16 ? 8 : K == 8 ? 12 : pow2 ? 16 : 24;
+    if (S < from) return S >= 5 && npix <= 128L * num_sms ? 32 : 1;
+    return S <= 20 ? 8 : 32;
 }
 
 cudaError_t glint_launch_probs(const glint_ctx *ctx, const glint_env *env, const glint_gbuffer *g,
@@ -164,8 +167,10 @@ cudaError_t glint_launch_probs(const glint_ctx *ctx, const glint_env *env, const
     a.p_out = p_out;
     const int ev = p->evaluator == GLINT_EVAL_E2 ? EV_E2 : p->evaluator == GLINT_EVAL_E1_ANISO ? EV_E1A : EV_E1;
     if (a.npix == 0) return cudaSuccess;
-    if (ev == EV_E2 && e2_by_warps(env->d.K, a.e2S, a.npix, ctx->num_sms))
-        return glint_launch_e2_probs(a, env->d.K, ctx->num_sms, s);
+    if (ev == EV_E2) {
+        const int lanes = e2_lanes(env->d.K, a.e2S, a.npix, ctx->num_sms);
+        if (lanes > 1) return glint_launch_e2_probs(a, env->d.K, lanes, ctx->num_sms, s);
+    }
     switch (env->d.K) {
     case 2: return launch_probs<2>(a, ev, s);
     case 4: return launch_probs<4>(a, ev, s);
