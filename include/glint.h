@@ -342,10 +342,17 @@ int glint_hostpipe_last_in_place(const glint_hostpipe *pipe);
 /* Reflection probabilities p_k (Eq. probhk) of every pixel of `gbuf` under
  * params->evaluator (E1, E2 or MLP; GIVEN is rejected; seed and count mode
  * are ignored), the
- * quantity glint_shade feeds to the counts.  p_out: device, width*height*K
- * floats, pixel-major; background pixels (N_0 <= 0) get 0.  Used to generate
- * the surrogate's training targets (E2) and to measure its error.  Enqueued on
- * `stream`. */
+ * quantity glint_shade feeds to the counts (E2: up to the rounding of its sums).
+ * p_out: device, width*height*K floats, pixel-major; background pixels (N_0 <=
+ * 0) get 0.  Used to generate the surrogate's training targets (E2) and to
+ * measure its error.  Enqueued on `stream`.
+ *
+ * E2 splits a pixel's S x S points over 1, 8 or 32 lanes and adds up in the order
+ * of the split; glint_shade always takes one lane.  A pixel's p_k therefore
+ * depends in its last bits on the split, which follows from K and S and, for S in
+ * [5, 8) at K = 16, [5, 12) at K = 8 and [5, 24) but 16 at K <= 4, from whether the
+ * frame has more than 128 pixels an SM: there a crop and its whole frame can differ
+ * so.  Each split is as close to the quadrature as the others. */
 glint_status glint_reflect_probs(glint_ctx *ctx, const glint_env *env, const glint_gbuffer *gbuf,
                                  const glint_params *params, float *p_out, void *stream);
 

@@ -153,7 +153,8 @@ cudaError_t glint_launch_shade(const glint_ctx *ctx, const glint_env *env, const
 // lanes: 64 x 64 43 / 24 us, 1280 x 720 3514 / 3598; S = 16 21 / 14, 1597 / 1710).
 // Below those S frames that leave most of the chip without a thread of its own
 // take 32 lanes (160 x 120, K = 8, thread / 32 lanes: S = 4 15 / 16 us, S = 5 22 / 17, S = 11
-// 93 / 30).  The splits differ in rounding.
+// 93 / 30).  The splits differ in rounding (include/glint.h says so): this is the
+// one choice by the frame's size.
 static int e2_lanes(int K, int S, long npix, int num_sms) {
     const bool pow2 = (S & (S - 1)) == 0;
     const int from = K == 16 ? 8 : K == 8 ? 12 : pow2 ? 16 : 24;
