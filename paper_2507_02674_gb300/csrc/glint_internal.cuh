@@ -290,7 +290,8 @@ __device__ __forceinline__ void pdl_wait_then_release_few() {
 }
 
 // A launch whose blocks may start while the stream's previous kernel runs
-// (pdl), or an ordinary one.
+// (pdl), or an ordinary one.  Returns and clears a launch error, as
+// cudaGetLastError() after a launch does.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
                        Args... args) {
@@ -304,12 +305,14 @@ cudaError_t launch_pdl(bool pdl, void (*kernel)(KArgs...), unsigned grid, unsign
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here, not by a later call once more
+    return e;
 }
 
 }  // namespace glint
 
-// Launchers implemented in the .cu files (return cudaGetLastError()).
+// Launchers implemented in the .cu files (return, and clear, the launch's error).
 cudaError_t glint_launch_lut(float4 *lut, int n, int q, cudaStream_t s);
 cudaError_t glint_launch_env(glint_env *env, const void *texels, cudaStream_t s, int *launches);
 cudaError_t glint_launch_filter_table(glint_env *env, cudaStream_t s);
