@@ -266,8 +266,10 @@ __device__ __forceinline__ void draw_single_real(float N, const NodeParams &np, 
     const bool open = (xi1c > Pnone) && (old || xi1 < N * np.p);
     n = 0.f;
     if (open) {
-        const float mu = 1.f + (N - 1.f) * np.p;
-        const float sigma = fast_sqrt(fmaxf((N - 1.f) * np.p * np.q, 0.f));
+        // (written out: a kernel with the intermediates and one without round alike)
+        const float m = __fmul_rn(N - 1.f, np.p);
+        const float mu = __fadd_rn(1.f, m);
+        const float sigma = fast_sqrt(fmaxf(__fmul_rn(m, np.q), 0.f));
         const float z = hash_quantile(hash_uniform(h2));
         const float g = fminf(fmaxf(fmaf(sigma, z, mu), 1.f), fmaxf(N, 1.f));
         n = old ? floorf(g) : g;
