@@ -591,8 +591,8 @@ size_t glint_arena_largest_free(const glint_arena *arena);
  * pixels ending at multiples of tile_pixels (or the frame's end): first one
  * item for every unfinished frame, so that every admitted frame progresses in
  * every tick, then items for the frames with the fewest pixels left (frame
- * order among equals) until tick_pixels are planned; at most max_items in all.  Writes the items, advances next[] and returns the item
- * count. */
+ * order among equals) until tick_pixels are planned; at most max_items in all.
+ * Writes the items, advances next[] and returns the item count. */
 int glint_plan_tick(long *next, const long *npix, int nframes, long tick_pixels, int tile_pixels, int *item_frame,
                     long *item_first, int *item_count, int max_items);
 

@@ -773,7 +773,7 @@ static void filtered_at(const double *pref, int R, const int *widths, int C, dou
 /* --------------------------------------------------------------------------
  * Anisotropic E1 by multi-tap prefiltered look-ups (the multiple filtered
  * look-ups along an anisotropic lobe that the paper's related work and its
- * limitations section point to for anisotropic materials; SURVEY NEXT-1).
+ * limitations section point to for anisotropic materials).
  * Reading: the lobe of reflected directions w_i is taken as an ellipse whose
  * axes are the images of the slope axes t and b: J_t a_x and J_b a_y, with
  * J_t = 2 (-(w_o.t) n - mu_o t), J_b likewise, the derivatives of the mirror

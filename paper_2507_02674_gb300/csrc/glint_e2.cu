@@ -153,7 +153,8 @@ __device__ __forceinline__ void add_texel(const float4 *__restrict__ lev, unsign
 // six (80 registers) where it is faster (8 lanes, rough, K = 8: S = 16 1705 -> 1597 us,
 // but S = 24 3515 -> 3596; K = 16: S = 16 3116 -> 2967, S = 24 7020 -> 6687).
 template <int K, bool FIXED, int G>
-__global__ void __launch_bounds__(kWarps * 32, G == 8 && (FIXED || K == 16) ? 6 : 5) k_e2_probs(ShadeArgs a, int steps) {
+__global__ void __launch_bounds__(kWarps * 32, G == 8 && (FIXED || K == 16) ? 6 : 5) k_e2_probs(ShadeArgs a,
+                                                                                                int steps) {
     constexpr int KW4 = (3 + K + 3) / 4 - 1, kGroups = 32 / G, kMaxPpw = kGroups * kMaxSteps;
     static_assert(kMaxPpw <= 32, "a warp's pixels are staged by a lane each");
     __shared__ float2 ring[kMaxS];   // r, 2 s
@@ -306,7 +307,8 @@ __global__ void __launch_bounds__(kWarps * 32, G == 8 && (FIXED || K == 16) ? 6 
             }
         }
         group_sums<K, G>(acc);
-        constexpr int kPer = G >= K ? G / K : 1, kOwn = G >= K ? 1 : K / G;  // lanes that hold the same sum, sums a lane
+        constexpr int kPer = G >= K ? G / K : 1;  // lanes that hold the same sum
+        constexpr int kOwn = G >= K ? 1 : K / G;  // sums a lane holds
         if (q < a.npix && lane % G % kPer == 0) {
 #pragma unroll
             for (int i = 0; i < kOwn; ++i) {

@@ -18,8 +18,8 @@
 // accumulator fragments of two adjacent n-tiles are exactly the A fragment of
 // the next layer's k-step, so activations stay in registers between layers
 // (ReLU and BF16 rounding applied on the way).  The inference and forward
-// kernels are persistent: each block stages the weights in shared memory once
-// and loops over 128-row tiles.
+// kernels are persistent: each block stages the weights in shared memory once,
+// and its warps loop over tiles of 32 rows (inference over 128 pixels a block).
 #include <cuda_bf16.h>
 
 #include <stdio.h>
@@ -62,12 +62,6 @@ __device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], uint32
 }
 
 __device__ __forceinline__ uint32_t ld32(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
-
-__device__ __forceinline__ uint32_t pair16(const __nv_bfloat16 *lo, const __nv_bfloat16 *hi) {
-    const uint32_t a = *reinterpret_cast<const uint16_t *>(lo);
-    const uint32_t b = *reinterpret_cast<const uint16_t *>(hi);
-    return a | (b << 16);
-}
 
 // Every [rows][64] BF16 tile in shared memory (inputs, activations,
 // backpropagated signals and the 64-wide weight matrices) is stored with its
@@ -739,9 +733,9 @@ __global__ void __launch_bounds__(kNT) k_mlp_features(ShadeArgs a, uint4 *__rest
 // b, b + G, b + 2G, ... (G = gridDim.x) of the batch and accumulates its
 // gradient (each sample's loss weighted by 1/batch) in partial[b][kP], always
 // in the same order, so the result does not depend on scheduling; its summed
-// squared error sum_k (p_k - y_k)^2 goes to loss[b].  A chunk of 32 samples gives a batch of 8192
-// 256 blocks, so every SM has work; the 16-row tiles of the chunk go to the
-// warps in turn.
+// squared error sum_k (p_k - y_k)^2 goes to loss[b].  A chunk of 32 samples gives
+// a batch of 8192 256 blocks, so every SM has work; a warp takes one of the
+// chunk's two 16-row tiles and half of a layer's outputs.
 constexpr int kChunk = 32;
 static_assert(kChunk * 8 % 128 == 0, "whole 16-byte pieces of inputs per thread");
 

@@ -101,8 +101,8 @@ cudaError_t launch_k(const ShadeArgs &args, bool integer, bool debug, int ev, cu
 template <int K>
 cudaError_t launch_probs(const ShadeArgs &args, int ev, cudaStream_t s) {
     const unsigned grid = (unsigned)((args.npix + kShadeNT - 1) / kShadeNT);
-    return launch_pdl(true, ev == EV_E2 ? k_probs<K, EV_E2> : ev == EV_E1A ? k_probs<K, EV_E1A> : k_probs<K, EV_E1>, grid,
-                      kShadeNT, 0, s, args);
+    auto kernel = ev == EV_E2 ? k_probs<K, EV_E2> : ev == EV_E1A ? k_probs<K, EV_E1A> : k_probs<K, EV_E1>;
+    return launch_pdl(true, kernel, grid, kShadeNT, 0, s, args);
 }
 
 }  // namespace

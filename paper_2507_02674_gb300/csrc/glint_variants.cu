@@ -23,10 +23,9 @@ __global__ void __launch_bounds__(kShadeNT, shade_min_blocks(K)) k_shade_var(Sha
 template <int K, int DRAW, int GRID>
 cudaError_t launch_kd(const ShadeArgs &a, bool integer, bool debug, cudaStream_t s) {
     const unsigned grid = (unsigned)((a.npix + kShadeNT - 1) / kShadeNT);
-    return launch_pdl(true,
-                      integer ? (debug ? k_shade_var<K, true, true, DRAW, GRID> : k_shade_var<K, true, false, DRAW, GRID>)
-                              : (debug ? k_shade_var<K, false, true, DRAW, GRID> : k_shade_var<K, false, false, DRAW, GRID>),
-                      grid, kShadeNT, 0, s, a);
+    auto kernel = integer ? (debug ? k_shade_var<K, true, true, DRAW, GRID> : k_shade_var<K, true, false, DRAW, GRID>)
+                          : (debug ? k_shade_var<K, false, true, DRAW, GRID> : k_shade_var<K, false, false, DRAW, GRID>);
+    return launch_pdl(true, kernel, grid, kShadeNT, 0, s, a);
 }
 
 template <int K>
@@ -39,7 +38,8 @@ cudaError_t launch_k(const ShadeArgs &a, bool integer, bool debug, int draw, int
 
 }  // namespace
 
-cudaError_t glint_launch_shade_variant(const ShadeArgs &a, int K, bool integer, bool debug, int draw, int grid, cudaStream_t s) {
+cudaError_t glint_launch_shade_variant(const ShadeArgs &a, int K, bool integer, bool debug, int draw, int grid,
+                                       cudaStream_t s) {
     if (a.npix == 0) return cudaSuccess;
     switch (K) {
     case 2: return launch_k<2>(a, integer, debug, draw, grid, s);
