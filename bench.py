@@ -383,7 +383,7 @@ def surrogate(args, glint, render, ctx, fr, gb, planes, out, stream, flush, seed
     ms_e1a = timed(e1a_step, args.steps)
     ms_e2 = timed(e2_step, max(3, min(args.steps, 10)))
     return {
-        "path": "env update + glint_shade with the surrogate fused in (per 256-pixel block: inputs, BF16 "
+        "path": "env update + glint_shade with the surrogate fused in (per warp of 32 pixels: inputs, BF16 "
                 "mma.sync network, draws with its p_k from shared memory; one launch)",
         "value": round(npix / (float(ms_nn.mean()) / 1e3) / 1e6, 3), "unit": "Mpixel/s",
         "ms_per_step": round(float(ms_nn.mean()), 4),

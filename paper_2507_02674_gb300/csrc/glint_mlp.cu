@@ -369,7 +369,7 @@ __device__ __forceinline__ void net_tile(const SmemInfer &sm, long base, long n,
 // the next one on its way to shared memory (cp.async) while the network runs on
 // the current one; log-priors and results go straight between global memory and
 // the accumulator layout (8 bytes a lane, whole 32-byte rows a quad at K = 8).
-// Bound by the mma.sync pipe (51% busy, its throttle the largest stall) and the
+// Bound by the mma.sync pipe (50% busy, its throttle the largest stall) and the
 // chains of dependent products: 1,000,003 rows in 62.9 us, against 98.9 when a
 // block staged 128 rows, synchronised, and loaded every fragment in 32-bit
 // pieces for one 16-row tile.
