@@ -29,7 +29,7 @@
 // fourth ring instead of eight in a row 6.6; words exchanged through shared
 // memory 7.4; blocks of 12 or 24 warps in step 6.3 and 6.5; without the branch over
 // invalid points 6.9.  The sums of 8 lanes in the order of 32, so that both give the
-// same bits: K = 8, S = 13, smooth 977 us.)
+// same bits: K = 8, S = 13, smooth 985 us.)
 #include "glint_internal.cuh"
 #include "glint_probs.cuh"
 
